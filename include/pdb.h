@@ -115,7 +115,7 @@ typedef enum { PDB_LOSS_LOGISTIC = 0, PDB_LOSS_SQUARED = 1, PDB_LOSS_HINGE = 2 }
  *           most examples): one thread block runs the examples strictly in
  *           data order (Algorithm 1 itself), prefetching ids, values and
  *           weights ahead and forwarding each new weight whose next
- *           occurrence is among the next 16 examples through shared memory,
+ *           occurrence is among the next 40 examples through shared memory,
  *           so a dependency hop costs a few hundred cycles (examples of at
  *           most 256 ids).  Longer examples run with all n_cols weights
  *           resident in shared memory instead, when they fit (about 55,000
@@ -237,9 +237,9 @@ int pdb_conflicts_arrays(const pdb_conflicts *c, const int32_t **csc_pos, const 
  *     position waits for the version equal to its occurrence rank (the
  *     conflicts' gate array).
  *   CHAIN (Algorithm 1 in data order on one SM): per position, whether an
- *     example among the 16 before it writes its feature last (its weight is
+ *     example among the 40 before it writes its feature last (its weight is
  *     then forwarded on chip) and where the next occurrence sits if within
- *     the 16 examples after; nothing when the
+ *     the 40 examples after; nothing when the
  *     longest example has more than 256 ids and the weights fit in shared
  *     memory (resident); PDB_ETOOBIG when they do not.
  *   WINDOW: per feature a 64-bit hand-off record for near pairs, one

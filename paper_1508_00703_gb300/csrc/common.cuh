@@ -39,7 +39,7 @@ int block_ready_run(const pdb_csr *X, const float *y, const uint32_t *gate, floa
 int resident_run(const pdb_csr *X, const float *y, float *w, int loss, float eta, int epochs, int max_row,
                  int *status, uint64_t *trace, cudaStream_t s);
 int chain_schedule(const int32_t *prev, const int32_t *next, const int32_t *row_of, const int64_t *row_ptr,
-                   int64_t nnz, int64_t max_row, uint32_t *link, const int *status, cudaStream_t s);
+                   int64_t nnz, uint32_t *link, const int *status, cudaStream_t s);
 int chain_run(const pdb_csr *X, const float *y, const uint32_t *link, float *w, int loss, float eta, int epochs,
               int max_row, int *status, uint64_t *trace, cudaStream_t s);
 void note_launch();                                   // count one kernel launch (pdb_launch_count)
@@ -240,16 +240,33 @@ __device__ __forceinline__ float dev_grad(int loss, float m, float y)
     return __fmul_rn(y, m) < 1.0f ? -y : 0.0f;
 }
 
-// the step size times the derivative, eta * dev_grad(loss, m, y), with the
-// same bits: on the reciprocal path eta * (-y q) = (-y eta) * q exactly, so
-// the sign goes on eta, which is known before m
-__device__ __forceinline__ float dev_step(int loss, float m, float y, float eta)
+// The step size times the derivative, eta * dev_grad(loss, m, y), with the
+// same bits, no branch and a shorter dependent path from m; `redo` is set
+// where that does not hold and the general form must be taken.  For the
+// logistic loss with y = +1 or -1 and -2^21 < y m <= 87 the exponential's
+// pieces fold: y rides on log2e and on eta (sign changes are exact);
+// e = exp(y m) is only needed in 1 + e, so below the normal range, where
+// 1 + e = 1, any tiny value stands for it (k is held at -126 and p stays
+// between 0.5 and 2: |y m log2e| < 2^22); and above it no scaling overflows.
+__device__ __forceinline__ float dev_step_fast(int loss, float m, float y, float eta, bool &redo)
 {
     if (loss == PDB_LOSS_LOGISTIC) {
-        const float d = __fadd_rn(1.0f, dev_expf(__fmul_rn(y, m)));
-        float c = __fmul_rn(y > 0.0f ? -eta : eta, recip_ge1(d));
-        if (!((y == 1.0f || y == -1.0f) && d < 0x1p126f)) c = __fmul_rn(eta, __fdiv_rn(-y, d));
-        return c;
+        const float x = __fmul_rn(y, m);
+        const float u = __fadd_rn(__fmul_rn(m, __fmul_rn(y, 1.44269502162933349609375f)), 12582912.0f);
+        const float kf = __fsub_rn(u, 12582912.0f);
+        const int k = max(__float_as_int(u) - 0x4B400000, -126);
+        const float r = __fsub_rn(__fmaf_rn(-kf, 0.693145751953125f, x), __fmul_rn(kf, 1.428606765330187045e-06f));
+        float p = 1.0f / 5040.0f;
+        p = __fmaf_rn(p, r, 1.0f / 720.0f);
+        p = __fmaf_rn(p, r, 1.0f / 120.0f);
+        p = __fmaf_rn(p, r, 1.0f / 24.0f);
+        p = __fmaf_rn(p, r, 1.0f / 6.0f);
+        p = __fmaf_rn(p, r, 0.5f);
+        p = __fmaf_rn(p, r, 1.0f);
+        p = __fmaf_rn(p, r, 1.0f);
+        const float d = __fadd_rn(1.0f, __fmul_rn(p, __int_as_float((k + 127) << 23)));
+        redo |= !((y == 1.0f || y == -1.0f) && x <= 87.0f && x > -0x1p21f);
+        return __fmul_rn(y > 0.0f ? -eta : eta, recip_ge1(d));
     }
     return __fmul_rn(eta, dev_grad(loss, m, y));
 }
