@@ -38,6 +38,9 @@ int block_ready_run(const pdb_csr *X, const float *y, const uint32_t *gate, floa
                     int epochs, int max_row, int *status, uint64_t timeout, uint64_t *trace, cudaStream_t s);
 int resident_run(const pdb_csr *X, const float *y, float *w, int loss, float eta, int epochs, int max_row,
                  int *status, uint64_t *trace, cudaStream_t s);
+bool dense_fits(int64_t n_rows, int64_t n_cols, int64_t nnz, int64_t max_row, bool ascending);   // dense.cu
+int dense_run(const pdb_csr *X, const float *y, float *w, int loss, float eta, int epochs, const int *status,
+              uint64_t *trace, cudaStream_t s);
 int chain_schedule(const int32_t *prev, const int32_t *next, const int32_t *row_of, const int64_t *row_ptr,
                    int64_t nnz, uint32_t *link, const int *status, cudaStream_t s);
 int chain_run(const pdb_csr *X, const float *y, const uint32_t *link, float *w, int loss, float eta, int epochs,
@@ -359,6 +362,7 @@ struct pdb_schedule {
                               // under prefix gates the known-done prefix of each feature's reads / writes
     unsigned *rbits, *wbits;  // READY under pdb_ssp_epoch with prefix gates: done-bitmaps over the CSC slots
     uint32_t *link;           // CHAIN: per position, receive flag and push target
+    bool dense;               // CHAIN: every example holds every feature (weights in registers, no link words)
     bool resident;            // CHAIN: weights resident in shared memory (no link words)
     unsigned epochs_run;      // WINDOW: epochs run so far (epoch stamp of the record tags, done-flag tag)
     unsigned *prog;           // WINDOW: done flag per chunk of examples (zeroed once)
