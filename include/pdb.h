@@ -327,8 +327,10 @@ int pdb_ssp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, cons
  * dloss/dm at the weights of the batch start (read barrier), then each
  * feature j takes delta_j = sum over the batch's examples, ascending, of
  * c_i * x_ij and w_j = w_j - delta_j (write barrier).  batch = 1 equals
- * sequential SGD (Theorem 1).  Allocates per-call scratch stream-ordered;
- * sizing it waits (host) for the conflict build of c to finish. */
+ * sequential SGD (Theorem 1).  Two kernel launches per batch (no wait inside a
+ * kernel: opts->blocks_per_sm and wait_timeout_s play no part).  Allocates
+ * per-call scratch stream-ordered and waits (host) for the conflict build of c
+ * to finish. */
 int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, float *w, pdb_loss loss, float eta,
                   int64_t batch, int n_epochs, const pdb_opts *opts, void *stream);
 

@@ -22,7 +22,7 @@ struct Launch {
 };
 Launch launch_info();
 int occupancy_blocks(const void *kernel, int threads, size_t smem);
-int persistent_grid(const void *kernel, const pdb_opts *opts);
+int persistent_grid(const void *kernel, const pdb_opts *opts, int threads = THREADS);
 uint64_t timeout_ns(const pdb_opts *opts);
 int alloc(void **p, size_t bytes, cudaStream_t s);   // stream-ordered, 256-byte aligned
 void release(void *p, cudaStream_t s);
@@ -386,6 +386,8 @@ struct pdb_bsp_plan {
     int32_t *bcol, *brow;
     cudaEvent_t ev_use;       // recorded after the last work any call enqueued on the plan
     float *bval;
+    int32_t *runs;            // first pairs of each batch's runs (same feature)
+    uint2 *n_runs;            // [n_batches] short and long runs
 };
 
 namespace pdb {

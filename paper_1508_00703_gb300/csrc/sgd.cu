@@ -302,7 +302,33 @@ __global__ void k_unpack(const unsigned long long *__restrict__ rec, int64_t n, 
 }
 
 // ---------------------------------------------------------------- BSP
-// margin of example t at the current w (all lanes return the same value)
+// Per batch two launches: k_bsp_coef (the reads) and k_bsp_apply (the writes).
+// A batch's launches follow each other with programmatic dependence: a kernel
+// starts while the one before it drains, reads what no batch writes (row
+// bounds, ids, values, rows of pairs), and waits here before it reads what the
+// one before wrote.  Without that launch attribute both are no-ops.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// loads that stay where they are written: the compiler may move a load of
+// read-only data down to its use, behind the work that should hide it
+__device__ __forceinline__ int32_t ld_here(const int32_t *p)
+{
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_here(const float *p)
+{
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// margin of example t at the current w (all lanes return the same value); rows
+// longer than 32 ids load BSP_M elements per lane at a time, the next ones' ids
+// and values while these ones' weights are on their way
+constexpr int BSP_M = 8;
 __device__ __forceinline__ float margin(int t, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
                                         const float *__restrict__ val, const float *w)
 {
@@ -310,166 +336,260 @@ __device__ __forceinline__ float margin(int t, const int64_t *__restrict__ row_p
     const int64_t b = row_ptr[t];
     const int k = (int)(row_ptr[t + 1] - b);
     float acc = 0.0f;
-    for (int i = lane; i < k; i += 32) acc = __fmaf_rn(__ldcg(w + col[b + i]), val ? val[b + i] : 1.0f, acc);
+    if (k <= 32) {
+        int j0 = 0;
+        float x0 = 1.0f;
+        if (lane < k) {
+            j0 = ld_here(col + b + lane);
+            if (val) x0 = ld_here(val + b + lane);
+        }
+        wait_previous();
+        if (lane < k) acc = __fmaf_rn(__ldcg(w + j0), x0, acc);
+        return warp_combine(acc);
+    }
+    int j[BSP_M];
+    float x[BSP_M], wv[BSP_M], xc[BSP_M];
+    auto load = [&](int base) {
+#pragma unroll
+        for (int u = 0; u < BSP_M; ++u) {
+            const int i = min(base + 32 * u + lane, k - 1);      // past the end: the last element, not added
+            j[u] = ld_here(col + b + i);
+            x[u] = val ? ld_here(val + b + i) : 1.0f;
+        }
+    };
+    load(0);
+    wait_previous();
+    for (int base = 0; base < k; base += 32 * BSP_M) {
+#pragma unroll
+        for (int u = 0; u < BSP_M; ++u) {
+            wv[u] = __ldcg(w + j[u]);
+            xc[u] = x[u];
+        }
+        if (base + 32 * BSP_M < k) load(base + 32 * BSP_M);
+#pragma unroll
+        for (int u = 0; u < BSP_M; ++u)
+            if (base + 32 * u + lane < k) acc = __fmaf_rn(wv[u], xc[u], acc);
+    }
     return warp_combine(acc);
 }
 
-// The next CH terms of feature j's run from q (the batch's sorted pairs end at
-// s1, its products start at s0), added to delta in ascending example order.
-// Loads first, then the dependent adds.  Returns whether the run continues
-// past the chunk (q then points after it).
-template <int CH>
-__device__ __forceinline__ bool run_chunk_prod(int32_t j, int64_t &q, int64_t s0, int64_t s1,
-                                               const int32_t *__restrict__ bcol, const float *prod, float &delta)
+// The write half of a batch works on its pairs [s0, s1), sorted by (feature,
+// example): feature j's terms c_i * x_ij form one run, added in ascending
+// example order from +0; then w_j = w_j - sum.  The batch's rows start at r0
+// and coef holds their coefficients.  Positions are below 2^31; unsigned, so
+// that looking some turns ahead does not overflow.
+struct BspPairs {
+    uint32_t s1;            // the batch's end
+    int32_t r0, rows;
+    const int32_t *__restrict__ col, *__restrict__ row;
+    const float *__restrict__ val;
+    const float *coef;
+};
+
+// the coefficient of a pair's example (`bad` set for a row outside the batch:
+// cannot happen with a consistent batch sort)
+__device__ __forceinline__ float bsp_coef_of(const BspPairs &P, int32_t row, bool &bad)
 {
-    int32_t jj[CH];
-    float pp[CH];
+    const int32_t i = row - P.r0;
+    const bool in = i >= 0 && i < P.rows;
+    bad |= !in;
+    return ld_here(P.coef + (in ? i : 0));
+}
+
+// A run longer than BSP_LONG terms is summed by a block: warp 0 adds, the
+// others make the products.
+constexpr int BSP_LONG = 16;
+constexpr int BSP_THREADS = 128;
+constexpr int BSP_BLOCKS = 8;                       // per SM
+constexpr int BSP_U = 8;                            // terms per producing thread and stage
+constexpr int BSP_STAGE = (BSP_THREADS - 32) * BSP_U;
+constexpr int BSP_ADDS = 192;                       // terms the adding warp takes between two loop branches
+
+// The sum of the `len` terms from pair q on, by the whole block; the result is
+// warp 0's.  The sum is a chain of dependent additions (4 cycles each), so one
+// warp does nothing else: it adds a stage of products from shared memory, 16
+// bytes per load, every lane the same, while the other warps form the next
+// stage's (rows loaded one stage earlier still).  A stage's terms past the
+// run's end are -0, which changes no sum.
+__device__ __forceinline__ float block_run_sum(const BspPairs &P, uint32_t q, uint32_t len, float (*buf)[BSP_STAGE],
+                                               bool &bad)
+{
+    const int t = (int)threadIdx.x - 32;            // producer, < 0: the adding warp
+    const uint32_t end = q + len, stages = (len + BSP_STAGE - 1) / BSP_STAGE;
+    int32_t row[BSP_U];
+    auto rows_of = [&](uint32_t k) {
+#pragma unroll
+        for (int u = 0; u < BSP_U; ++u)
+            row[u] = ld_here(P.row + min(q + k * BSP_STAGE + u * (BSP_THREADS - 32) + t, end - 1));
+    };
+    auto produce = [&](uint32_t k) {                // stage k, its rows in row[]
+        float v[BSP_U], c[BSP_U];
+#pragma unroll
+        for (int u = 0; u < BSP_U; ++u)
+            v[u] = ld_here(P.val + min(q + k * BSP_STAGE + u * (BSP_THREADS - 32) + t, end - 1));
+        if (k == 0) wait_previous();                // the coefficients are the kernel before's
+#pragma unroll
+        for (int u = 0; u < BSP_U; ++u) c[u] = bsp_coef_of(P, row[u], bad);
+        if (k + 1 < stages) rows_of(k + 1);
+#pragma unroll
+        for (int u = 0; u < BSP_U; ++u) {
+            const int i = u * (BSP_THREADS - 32) + t;
+            buf[k & 1][i] = k * BSP_STAGE + i < len ? __fmul_rn(c[u], v[u]) : -0.0f;
+        }
+    };
+    float delta = 0.0f;
+    if (t >= 0) {
+        rows_of(0);
+        produce(0);
+    } else {
+        wait_previous();
+    }
+    __syncthreads();
+    for (uint32_t k = 0; k < stages; ++k) {
+        if (t >= 0) {
+            if (k + 1 < stages) produce(k + 1);
+        } else {
+            const float4 *b4 = reinterpret_cast<const float4 *>(buf[k & 1]);
+            const int n = (int)min(len - k * BSP_STAGE, (uint32_t)BSP_STAGE);
+#pragma unroll 1
+            for (int i = 0; i < n; i += BSP_ADDS, b4 += BSP_ADDS / 4)
+#pragma unroll
+                for (int e = 0; e < BSP_ADDS / 4; ++e) {
+                    const float4 f = b4[e];
+                    delta = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(delta, f.x), f.y), f.z), f.w);
+                }
+        }
+        __syncthreads();
+    }
+    return delta;
+}
+static_assert(BSP_STAGE % BSP_ADDS == 0, "the adding warp reads whole groups");
+
+// The next CH terms of feature j's run from q, added to delta (loads first,
+// then the dependent adds).  Returns whether the run may continue past them.
+template <int CH>
+__device__ __forceinline__ bool thread_run_chunk(const BspPairs &P, int32_t j, uint32_t &q, float &delta, bool &bad)
+{
+    int32_t jj[CH], rr[CH];
+    float xx[CH], cc[CH];
 #pragma unroll
     for (int u = 0; u < CH; ++u) {
-        const bool in = q + u < s1;
-        jj[u] = in ? bcol[q + u] : -1;
-        pp[u] = in ? __ldcg(prod + (q + u - s0)) : 0.0f;
+        const bool in = q + u < P.s1;
+        jj[u] = in ? P.col[q + u] : -1;
+        rr[u] = in ? P.row[q + u] : P.r0;
+        xx[u] = in ? P.val[q + u] : 0.0f;
     }
     bool more = true;
+    int n = 0;
 #pragma unroll
     for (int u = 0; u < CH; ++u) {
         more = more && jj[u] == j;
-        if (more) delta = __fadd_rn(delta, pp[u]);
+        n += more;
+        cc[u] = bsp_coef_of(P, rr[u], bad);
     }
+#pragma unroll
+    for (int u = 0; u < CH; ++u)
+        if (u < n) delta = __fadd_rn(delta, __fmul_rn(cc[u], xx[u]));
     q += CH;
     return more;
 }
 
-// Runs longer than this many terms are summed by a whole warp.
-constexpr int BSP_LONG = 16;
-
-// Feature j's run from q, summed by the whole warp: 32 terms per load, the
-// adds in ascending order on every lane (each lane ends with the same delta).
-__device__ __forceinline__ float warp_run_sum(int32_t j, int64_t q, int64_t s0, int64_t s1,
-                                              const int32_t *__restrict__ bcol, const float *prod)
+// The runs of every batch, in no particular order: their first pairs at
+// runs[bptr[b] ..] (at most BSP_LONG terms) and, for longer ones, the first pair
+// and the length, two words each, backwards from runs[bptr[b + 1] - 1] (a long
+// run has more than two pairs, so the two lists never meet); counts in n_runs[b]
+// (short, long; zeroed before).  skey: the batch of each pair (null: one batch).
+__global__ void k_bsp_runs(const uint32_t *__restrict__ skey, const int32_t *__restrict__ bcol,
+                           const int64_t *__restrict__ bptr, int64_t nnz, int32_t *__restrict__ runs, uint2 *n_runs,
+                           const int *status)
 {
+    if (read_status(status)) return;
+    constexpr int E = 8;                // 256 pairs per warp and reservation: one address takes few atomics
     const int lane = threadIdx.x & 31;
-    float delta = 0.0f;
-    int32_t jn = q + lane < s1 ? bcol[q + lane] : -1;
-    float pn = q + lane < s1 ? __ldcg(prod + (q + lane - s0)) : 0.0f;
-    for (;;) {
-        const float pc = pn;
-        const int n = __popc(__ballot_sync(FULL, jn == j));   // the run is a prefix of the 32
-        if (n == 32) {                                          // next 32 in flight during the adds
-            q += 32;
-            jn = q + lane < s1 ? bcol[q + lane] : -1;
-            pn = q + lane < s1 ? __ldcg(prod + (q + lane - s0)) : 0.0f;
-        }
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * E;
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane) * E; base < nnz; base += stride) {
+        int32_t j[E], before[E], far[E];
+        uint32_t bt[E], bt_before[E], bt_far[E];
 #pragma unroll
-        for (int u = 0; u < 32; ++u) {
-            const float v = __shfl_sync(FULL, pc, u);
-            if (u < n) delta = __fadd_rn(delta, v);
+        for (int e = 0; e < E; ++e) {
+            const int64_t s = base + 32 * e + lane, f = s + BSP_LONG;
+            j[e] = s < nnz ? bcol[s] : -1;
+            before[e] = s > 0 && s < nnz ? bcol[s - 1] : -1;
+            far[e] = f < nnz ? bcol[f] : -1;
+            bt[e] = s < nnz && skey ? skey[s] : 0u;
+            bt_before[e] = s > 0 && s < nnz && skey ? skey[s - 1] : 0u;
+            bt_far[e] = f < nnz && skey ? skey[f] : 0u;
         }
-        if (n < 32) return delta;
+        unsigned sm[E], lm[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const bool start = j[e] >= 0 && (before[e] != j[e] || bt_before[e] != bt[e]);
+            const bool is_long = start && far[e] == j[e] && bt_far[e] == bt[e];
+            sm[e] = __ballot_sync(FULL, start && !is_long);
+            lm[e] = __ballot_sync(FULL, is_long);
+        }
+        // the batches of these pairs, one after the other (nearly always one)
+        const uint32_t b_first = __shfl_sync(FULL, bt[0], 0);
+        uint32_t b_last = 0;
+        {
+            const int64_t last = min64(nnz, base + 32 * E) - 1;
+            b_last = skey ? skey[last] : 0u;
+        }
+        for (uint32_t bb = b_first; bb <= b_last; ++bb) {
+            int n_s = 0, n_l = 0;
+            unsigned ms[E], ml[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const unsigned mine = __ballot_sync(FULL, bt[e] == bb);
+                ms[e] = sm[e] & mine;
+                ml[e] = lm[e] & mine;
+                n_s += __popc(ms[e]);
+                n_l += __popc(ml[e]);
+            }
+            unsigned at_s = 0, at_l = 0;
+            if (lane == 0 && n_s) at_s = atomicAdd(&n_runs[bb].x, (unsigned)n_s);
+            if (lane == 0 && n_l) at_l = atomicAdd(&n_runs[bb].y, (unsigned)n_l);
+            at_s = __shfl_sync(FULL, at_s, 0);
+            at_l = __shfl_sync(FULL, at_l, 0);
+            const int64_t b0 = bptr[bb], b1 = bptr[bb + 1];
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int64_t s = base + 32 * e + lane;
+                if (ms[e] >> lane & 1u) runs[b0 + at_s + __popc(ms[e] & lanemask_lt())] = (int32_t)s;
+                if (ml[e] >> lane & 1u) {
+                    // the run's length: doubling steps, then a binary search (the batch's
+                    // pairs are sorted by feature)
+                    int64_t lo = s + BSP_LONG, step = BSP_LONG, hi = lo + step;      // bcol[lo] == j
+                    while (hi < b1 && bcol[hi] == j[e]) {
+                        lo = hi;
+                        step *= 2;
+                        hi = lo + step;
+                    }
+                    if (hi > b1) hi = b1;
+                    while (hi - lo > 1) {
+                        const int64_t mid = lo + ((hi - lo) >> 1);
+                        if (bcol[mid] == j[e])
+                            lo = mid;
+                        else
+                            hi = mid;
+                    }
+                    const int64_t at = b1 - 2 * ((int64_t)at_l + __popc(ml[e] & lanemask_lt()) + 1);
+                    runs[at] = (int32_t)s;
+                    runs[at + 1] = (int32_t)(lo + 1 - s);
+                }
+                at_s += __popc(ms[e]);
+                at_l += __popc(ml[e]);
+            }
+        }
     }
 }
 
-// Algorithm 2a with B examples per step: reads (the margins at the batch-start
-// weights), barrier; the products c_i * x_ij of the batch's pairs, which are
-// pre-sorted by (batch, feature, example), barrier; writes (each feature's
-// products summed in ascending example order, one run of the sorted pairs),
-// barrier.  A feature's run is summed by one thread, or by a whole warp when
-// it is longer than BSP_LONG terms.  Batches without such runs (has_long[b] =
-// 0) skip the products step: each thread forms its run's products itself.
-__global__ __launch_bounds__(THREADS, 8) void k_bsp(int32_t n_rows, int64_t batch, int64_t n_batches,
-                                                 const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                                                 const float *__restrict__ val, const float *__restrict__ y,
-                                                 const int64_t *__restrict__ bptr, const int32_t *__restrict__ bcol,
-                                                 const int32_t *__restrict__ brow, const float *__restrict__ bval,
-                                                 const uint8_t *__restrict__ has_long, float *cbuf, float *prod,
-                                                 float *w, int loss, float eta, int epochs,
-                                                 GridBarrier *bar, int *status, uint64_t timeout)
-{
-    if (read_status(status)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthr = (int64_t)gridDim.x * blockDim.x;
-    const int gw = (int)(gtid >> 5), nw = (int)(nthr >> 5);
-    for (int ep = 0; ep < epochs; ++ep)
-        for (int64_t bi = 0; bi < n_batches; ++bi) {
-            const int64_t r0 = bi * batch, r1 = min64(n_rows, r0 + batch);
-            for (int64_t t = r0 + gw; t < r1; t += nw) {
-                float m = margin((int)t, row_ptr, col, val, w);
-                if (lane == 0) cbuf[t - r0] = __fmul_rn(eta, dev_grad(loss, m, y[t]));
-            }
-            if (!grid_sync(bar, status, timeout)) return;
-            const int64_t s0 = bptr[bi], s1 = bptr[bi + 1];
-            if (!has_long[bi]) {
-                // every run is short: one thread per run, term by term
-                for (int64_t s = s0 + gtid; s < s1; s += nthr) {
-                    const int32_t j = bcol[s];
-                    if (s > s0 && bcol[s - 1] == j) continue;
-                    float delta = 0.0f;
-                    for (int64_t q = s; q < s1 && bcol[q] == j; ++q) {
-                        const int64_t i = brow[q] - r0;
-                        if (i < 0 || i >= r1 - r0) {     // cannot happen with a consistent batch sort
-                            set_status(status, PDB_EFAULT);
-                            break;
-                        }
-                        delta = __fadd_rn(delta, __fmul_rn(__ldcg(cbuf + i), bval[q]));
-                    }
-                    __stcg(w + j, __fsub_rn(__ldcg(w + j), delta));
-                }
-                if (!grid_sync(bar, status, timeout)) return;
-                continue;
-            }
-            for (int64_t s = s0 + gtid; s < s1; s += nthr) {
-                int64_t i = brow[s] - r0;
-                if (i < 0 || i >= r1 - r0) {     // cannot happen with a consistent batch sort
-                    set_status(status, PDB_EFAULT);
-                    i = 0;
-                }
-                __stcg(prod + (s - s0), __fmul_rn(__ldcg(cbuf + i), bval[s]));
-            }
-            if (!grid_sync(bar, status, timeout)) return;
-            for (int64_t base = s0 + (int64_t)gw * 32; base < s1; base += (int64_t)nw * 32) {
-                const int64_t s = base + lane;
-                const int32_t j = s < s1 ? bcol[s] : -1;
-                const bool start = s < s1 && (s == s0 || bcol[s - 1] != j);
-                const bool is_long = start && s + BSP_LONG < s1 && bcol[s + BSP_LONG] == j;
-                if (start && !is_long) {
-                    // at most BSP_LONG terms: a short first chunk (most runs hold one or two)
-                    float delta = 0.0f;
-                    int64_t q = s;
-                    if (run_chunk_prod<2>(j, q, s0, s1, bcol, prod, delta) &&
-                        run_chunk_prod<8>(j, q, s0, s1, bcol, prod, delta))
-                        run_chunk_prod<8>(j, q, s0, s1, bcol, prod, delta);
-                    __stcg(w + j, __fsub_rn(__ldcg(w + j), delta));
-                }
-                for (unsigned lm = __ballot_sync(FULL, is_long); lm; lm &= lm - 1) {
-                    const int src = __ffs(lm) - 1;
-                    const int64_t sr = __shfl_sync(FULL, s, src);
-                    const int32_t jr = __shfl_sync(FULL, j, src);
-                    const float delta = warp_run_sum(jr, sr, s0, s1, bcol, prod);
-                    if (lane == 0) __stcg(w + jr, __fsub_rn(__ldcg(w + jr), delta));
-                }
-            }
-            if (!grid_sync(bar, status, timeout)) return;
-        }
-}
-
-// has_long[b] = 1 when batch b holds a feature run longer than BSP_LONG terms
-// (skey: batch of each pair in the (batch, feature, example) order)
-__global__ void k_bsp_long(const uint32_t *__restrict__ skey, const int32_t *__restrict__ bcol, int64_t nnz,
-                           uint8_t *__restrict__ has_long, const int *status)
-{
-    if (read_status(status)) return;
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s + BSP_LONG < nnz;
-         s += (int64_t)gridDim.x * blockDim.x)
-        if (bcol[s + BSP_LONG] == bcol[s] && skey[s + BSP_LONG] == skey[s]) has_long[skey[s]] = 1;
-}
-
 __global__ void k_bsp_keys(const int32_t *__restrict__ csc_pos, const int32_t *__restrict__ row_of, int64_t nnz,
-                           int64_t batch, uint32_t *__restrict__ key, const int *status)
+                           uint32_t batch, uint32_t *__restrict__ key, const int *status)
 {
     if (read_status(status)) return;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < nnz; s += (int64_t)gridDim.x * blockDim.x)
-        key[s] = (uint32_t)(row_of[csc_pos[s]] / batch);
+        key[s] = (uint32_t)row_of[csc_pos[s]] / batch;
 }
 
 __global__ void k_bsp_gather(const int32_t *__restrict__ bpos, const int32_t *__restrict__ col,
@@ -486,79 +606,78 @@ __global__ void k_bsp_gather(const int32_t *__restrict__ bpos, const int32_t *__
     }
 }
 
+__global__ void k_bsp_one_batch(int64_t *__restrict__ bptr, int64_t nnz)
+{
+    bptr[0] = 0;
+    bptr[1] = nnz;
+}
+
 // ---- Algorithm 2a split over data-parallel ranks (pdb_bsp_plan / coef / apply)
 // c_i = eta * dloss/dm(m_i(w), y_i) for the rows [r0, r1), one warp per example,
 // w the weights of the batch start (the read half of the step)
-__global__ void k_bsp_coef(int64_t r0, int64_t r1, const int64_t *__restrict__ row_ptr,
+__global__ __launch_bounds__(256, 5) void k_bsp_coef(int64_t r0, int64_t r1, const int64_t *__restrict__ row_ptr,
                            const int32_t *__restrict__ col, const float *__restrict__ val,
                            const float *__restrict__ y, const float *w, int loss, float eta, float *__restrict__ coef,
                            const int *status)
 {
+    launch_next();
     if (read_status(status)) return;
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t t = r0 + gw; t < r1; t += nw) {
-        const float m = margin((int)t, row_ptr, col, val, w);
-        if (lane == 0) coef[t - r0] = __fmul_rn(eta, dev_grad(loss, m, y[t]));
+        const float yt = y[t];
+        const float m = margin((int)t, row_ptr, col, val, w);       // waits for the batch before
+        if (lane == 0) coef[t - r0] = __fmul_rn(eta, dev_grad(loss, m, yt));
     }
 }
 
-// The write half of one batch: each feature's terms c_i * x_ij summed in
-// ascending example order from +0, then w_j = w_j - delta_j.  The batch's
-// pairs [s0, s1) are sorted by (feature, example); coef holds the whole
-// batch's coefficients (rows r0.. in order).  A run of at most BSP_LONG
-// terms is summed by one thread; a longer one by a whole warp, 32 terms per
-// load with the same adds in the same order on every lane.
-__global__ void k_bsp_apply(int64_t s0, int64_t s1, int64_t r0, int64_t rows, const int32_t *__restrict__ bcol,
-                            const int32_t *__restrict__ brow, const float *__restrict__ bval,
-                            const float *__restrict__ coef, float *w, int *status)
+// The write half of batch bi: coef holds the whole batch's coefficients (rows
+// r0.. in order).  Long runs one per block; short ones one per thread, on the
+// blocks without a long one when those are most.
+//
+// What bounds it: the longest run's additions (3000 terms of the hottest
+// feature in a batch of 4096 zipf(1.0) examples: ~6 us).  Measured, both
+// launches of such a batch: 12 us, against 41 in one cooperative kernel whose
+// warps loaded 32 terms, shuffled them out and added them before the next 32
+// arrived (27 cycles per term), with two grid barriers of ~3 us each; on 5000
+// dense examples of 960 features 37 us per batch against 113.  One warp doing
+// both loads and additions took 6 cycles per term alone and 13 with every SM
+// doing so.
+__global__ __launch_bounds__(BSP_THREADS, BSP_BLOCKS) void k_bsp_apply(
+    int64_t bi, const int64_t *__restrict__ bptr, int32_t r0, int32_t rows, const int32_t *__restrict__ bcol,
+    const int32_t *__restrict__ brow, const float *__restrict__ bval, const int32_t *__restrict__ runs,
+    const uint2 *__restrict__ n_runs, const float *coef, float *w, int *status)
 {
+    __shared__ __align__(16) float s_buf[2][BSP_STAGE];
+    launch_next();
     if (read_status(status)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t s0 = bptr[bi], s1 = bptr[bi + 1];
+    const uint2 n = n_runs[bi];
+    const BspPairs P = {(uint32_t)s1, r0, rows, bcol, brow, bval, coef};
     bool bad = false;
-    for (int64_t base = s0 + gw * 32; base < s1; base += nw * 32) {
-        const int64_t s = base + lane;
-        const int32_t j = s < s1 ? bcol[s] : -1;
-        const bool start = s < s1 && (s == s0 || bcol[s - 1] != j);
-        const bool is_long = start && s + BSP_LONG < s1 && bcol[s + BSP_LONG] == j;
-        if (start && !is_long) {
-            float delta = 0.0f;
-            for (int64_t q = s; q < s1 && bcol[q] == j; ++q) {
-                const int64_t i = brow[q] - r0;
-                bad |= i < 0 || i >= rows;
-                if (i >= 0 && i < rows) delta = __fadd_rn(delta, __fmul_rn(coef[i], bval[q]));
-            }
+    for (uint32_t i = blockIdx.x; i < n.y; i += gridDim.x) {
+        const int64_t at = s1 - 2 * ((int64_t)i + 1);
+        const uint32_t q = (uint32_t)runs[at], len = (uint32_t)runs[at + 1];
+        const float delta = block_run_sum(P, q, len, s_buf, bad);
+        if (threadIdx.x == 0) {
+            const int32_t j = bcol[q];
             w[j] = __fsub_rn(w[j], delta);
         }
-        for (unsigned lm = __ballot_sync(FULL, is_long); lm; lm &= lm - 1) {
-            const int src = __ffs(lm) - 1;
-            int64_t q = __shfl_sync(FULL, s, src);
-            const int32_t jr = __shfl_sync(FULL, j, src);
-            float delta = 0.0f;
-            for (;;) {
-                const bool in = q + lane < s1 && bcol[q + lane] == jr;
-                float pv = 0.0f;
-                if (in) {
-                    const int64_t i = brow[q + lane] - r0;
-                    bad |= i < 0 || i >= rows;
-                    if (i >= 0 && i < rows) pv = __fmul_rn(coef[i], bval[q + lane]);
-                }
-                const int n = __popc(__ballot_sync(FULL, in));   // the run is a prefix of the 32
-#pragma unroll
-                for (int u = 0; u < 32; ++u) {
-                    const float v = __shfl_sync(FULL, pv, u);
-                    if (u < n) delta = __fadd_rn(delta, v);
-                }
-                if (n < 32) break;
-                q += 32;
-            }
-            if (lane == 0) w[jr] = __fsub_rn(w[jr], delta);
-        }
     }
-    if (__any_sync(FULL, bad) && lane == 0) set_status(status, PDB_EFAULT);   // cannot happen with a consistent plan
+    wait_previous();
+    const uint32_t b0 = n.y < gridDim.x / 2 ? n.y : 0;
+    if (blockIdx.x >= b0)
+        for (uint32_t i = (blockIdx.x - b0) * BSP_THREADS + threadIdx.x; i < n.x; i += (gridDim.x - b0) * BSP_THREADS) {
+            // at most BSP_LONG terms: a short first chunk (most runs hold one or two)
+            uint32_t q = (uint32_t)runs[s0 + i];
+            const int32_t j = bcol[q];
+            float delta = 0.0f;
+            if (thread_run_chunk<2>(P, j, q, delta, bad))
+                while (thread_run_chunk<4>(P, j, q, delta, bad)) {}
+            w[j] = __fsub_rn(w[j], delta);
+        }
+    if (bad) set_status(status, PDB_EFAULT);   // cannot happen with a consistent batch order
 }
 
 __global__ void k_eval_grad(const float *__restrict__ m, const float *__restrict__ y, float *__restrict__ out,
@@ -586,6 +705,90 @@ int register_width(const pdb_conflicts *c)
     }
     const int longest = c->h_info[2];
     return longest <= 64 ? 2 : longest <= 128 ? 4 : 8;
+}
+
+// The pairs of c in (batch, feature, example) order: feature, example and value
+// of each, where each batch's pairs start, and each batch's runs (enqueued on
+// s).  The CSC order is already (feature, example), so a single batch needs no
+// sort.
+int bsp_sort(pdb_conflicts *c, const float *val, int64_t batch, int64_t n_batches, int32_t *bcol, int32_t *brow,
+             float *bval, int64_t *bptr, int32_t *runs, uint2 *n_runs, cudaStream_t s)
+{
+    const int64_t nnz = c->nnz;
+    const int rf = fill_words(n_runs, 0u, sizeof(uint2) * std::max<int64_t>(n_batches, 1), s);
+    if (rf != PDB_OK) return rf;
+    if (nnz == 0) return fill_words(bptr, 0u, sizeof(int64_t) * (n_batches + 1), s);
+    uint32_t *key = nullptr, *skey = nullptr, *tkey = nullptr;
+    int32_t *bpos = nullptr, *tval = nullptr;
+    int rc = ensure_row_of(c, s);
+    if (n_batches > 1) {
+        rc = rc ? rc : alloc((void **)&key, sizeof(uint32_t) * nnz, s);
+        rc = rc ? rc : alloc((void **)&skey, sizeof(uint32_t) * nnz, s);
+        rc = rc ? rc : alloc((void **)&tkey, sizeof(uint32_t) * nnz, s);
+        rc = rc ? rc : alloc((void **)&bpos, sizeof(int32_t) * nnz, s);
+        rc = rc ? rc : alloc((void **)&tval, sizeof(int32_t) * nnz, s);
+        if (rc == PDB_OK) {
+            k_bsp_keys<<<grid_1d(nnz), 256, 0, s>>>(c->csc_pos, c->row_of, nnz, (uint32_t)batch, key, c->status);
+            note_launch();
+            // stable by batch: inside a batch the feature-major CSC order survives
+            rc = radix_sort(key, c->csc_pos, skey, bpos, tkey, tval, nnz, bits_for(n_batches - 1), c->status, s);
+            rc = rc ? rc : segment_bounds(skey, nnz, n_batches, nullptr, bptr, c->status, s);
+        }
+    } else if (rc == PDB_OK) {
+        k_bsp_one_batch<<<1, 1, 0, s>>>(bptr, nnz);
+        note_launch();
+    }
+    if (rc == PDB_OK) {
+        k_bsp_gather<<<grid_1d(nnz), 256, 0, s>>>(bpos ? bpos : c->csc_pos, c->col, val, c->row_of, nnz, bcol, brow,
+                                                  bval, c->status);
+        note_launch();
+        k_bsp_runs<<<grid_1d((nnz + 7) / 8), 256, 0, s>>>(skey, bcol, bptr, nnz, runs, n_runs, c->status);
+        note_launch();
+        if (cudaPeekAtLastError() != cudaSuccess) rc = PDB_ECUDA;
+    }
+    for (void *q : {(void *)key, (void *)skey, (void *)tkey, (void *)bpos, (void *)tval}) release(q, s);
+    return rc;
+}
+
+// the two launches of a batch; `follow`: the launch before on this stream is
+// this batch's or the batch before's other one, and this kernel may start while
+// it drains (launch_next, wait_previous)
+struct BspLaunch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr = {};
+    BspLaunch(int64_t blocks, int threads, bool follow, cudaStream_t s)
+    {
+        cfg.gridDim = dim3((unsigned)blocks);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.stream = s;
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = follow ? 1 : 0;
+    }
+};
+int launch_coef(int64_t r0, int64_t r1, const pdb_csr *X, const float *y, const float *w, int loss, float eta,
+                float *coef, const int *status, bool follow, cudaStream_t s)
+{
+    const BspLaunch l(grid_1d((r1 - r0) * 32), 256, follow, s);
+    const cudaError_t e = cudaLaunchKernelEx(&l.cfg, k_bsp_coef, r0, r1, X->row_ptr, X->col, X->val, y, w, loss, eta,
+                                             coef, status);
+    note_launch();
+    return e == cudaSuccess ? PDB_OK : PDB_ECUDA;
+}
+// pairs: at least the number of the batch's pairs
+int launch_apply(int64_t bi, int64_t r0, int64_t rows, int64_t pairs, int sms, const int64_t *bptr, const int32_t *bcol,
+                 const int32_t *brow, const float *bval, const int32_t *runs, const uint2 *n_runs, const float *coef,
+                 float *w, int *status, bool follow, cudaStream_t s)
+{
+    // a long run holds more than BSP_LONG pairs, so this covers one block per long run up to the cap
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((pairs + BSP_LONG - 1) / BSP_LONG,
+                                                                  (int64_t)sms * BSP_BLOCKS));
+    const BspLaunch l(blocks, BSP_THREADS, follow, s);
+    const cudaError_t e = cudaLaunchKernelEx(&l.cfg, k_bsp_apply, bi, bptr, (int32_t)r0, (int32_t)rows, bcol, brow,
+                                             bval, runs, n_runs, coef, w, status);
+    note_launch();
+    return e == cudaSuccess ? PDB_OK : PDB_ECUDA;
 }
 
 int check_run(const pdb_csr *X, const float *y, const pdb_conflicts *c, const float *w, int loss, int epochs)
@@ -749,22 +952,18 @@ int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, floa
     cudaEventRecord(cm->ev_bsp0, s);
     if (N > 0 && n_epochs > 0) {
         const int64_t n_batches = (N + batch - 1) / batch;
-        uint32_t *key = nullptr, *skey = nullptr, *tkey = nullptr;
-        int32_t *bpos = nullptr, *tval = nullptr, *bcol = nullptr, *brow = nullptr;
-        float *bval = nullptr, *cbuf = nullptr, *prod = nullptr;
-        uint8_t *has_long = nullptr;
+        int32_t *bcol = nullptr, *brow = nullptr;
+        float *bval = nullptr, *cbuf = nullptr;
         int64_t *bptr = nullptr;
-        GridBarrier *bar = nullptr;
-        rc = alloc((void **)&key, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&skey, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&tkey, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&bpos, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&tval, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&bcol, sizeof(int32_t) * nnz, s);
+        int32_t *runs = nullptr;
+        uint2 *n_runs = nullptr;
+        rc = alloc((void **)&bcol, sizeof(int32_t) * nnz, s);
         rc = rc ? rc : alloc((void **)&brow, sizeof(int32_t) * nnz, s);
         rc = rc ? rc : alloc((void **)&bval, sizeof(float) * nnz, s);
         rc = rc ? rc : alloc((void **)&cbuf, sizeof(float) * batch, s);
-        // products of the largest batch: at most batch x (longest row) pairs
+        rc = rc ? rc : alloc((void **)&bptr, sizeof(int64_t) * (n_batches + 1), s);
+        rc = rc ? rc : alloc((void **)&runs, sizeof(int32_t) * nnz, s);
+        rc = rc ? rc : alloc((void **)&n_runs, sizeof(uint2) * n_batches, s);
         int64_t max_row = 0;
         if (rc == PDB_OK) {
             if (cudaEventSynchronize(c->ev1) != cudaSuccess) {
@@ -773,46 +972,19 @@ int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, floa
             }
             max_row = c->h_info[2];
         }
-        rc = rc ? rc : alloc((void **)&has_long, (size_t)n_batches, s);
-        rc = rc ? rc : alloc((void **)&prod, sizeof(float) * std::max<int64_t>(1, std::min<int64_t>(nnz, batch * max_row)), s);
-        rc = rc ? rc : alloc((void **)&bptr, sizeof(int64_t) * (n_batches + 1), s);
-        rc = rc ? rc : alloc((void **)&bar, sizeof(GridBarrier), s);
-        if (rc == PDB_OK) {
-            rc = fill_words(bar, 0u, sizeof(GridBarrier), s);
-            if (rc == PDB_OK && nnz > 0) rc = ensure_row_of(cm, s);
-            if (rc == PDB_OK && nnz > 0) {
-                k_bsp_keys<<<grid_1d(nnz), 256, 0, s>>>(c->csc_pos, c->row_of, nnz, batch, key, cm->status); note_launch();
-                // stable by batch: inside a batch the feature-major CSC order survives
-                rc = radix_sort(key, c->csc_pos, skey, bpos, tkey, tval, nnz, bits_for(n_batches - 1), cm->status, s);
-                if (rc == PDB_OK)
-                    k_bsp_gather<<<grid_1d(nnz), 256, 0, s>>>(bpos, X->col, X->val, c->row_of, nnz, bcol, brow, bval,
-                                                              cm->status); note_launch();
+        rc = rc ? rc : bsp_sort(cm, X->val, batch, n_batches, bcol, brow, bval, bptr, runs, n_runs, s);
+        const int sms = launch_info().sms;
+        // the first launch waits for everything before it; the others start early
+        for (int ep = 0; rc == PDB_OK && ep < n_epochs; ++ep)
+            for (int64_t b = 0; rc == PDB_OK && b < n_batches; ++b) {
+                const int64_t r0 = b * batch, r1 = std::min(N, r0 + batch);
+                rc = launch_coef(r0, r1, X, y, w, (int)loss, eta, cbuf, cm->status, ep > 0 || b > 0, s);
+                if (rc == PDB_OK && nnz > 0)
+                    rc = launch_apply(b, r0, r1 - r0, std::min(nnz, (r1 - r0) * max_row), sms, bptr, bcol, brow, bval,
+                                      runs, n_runs, cbuf, w, cm->status, true, s);
             }
-            if (rc == PDB_OK) rc = segment_bounds(skey, nnz, n_batches, nullptr, bptr, cm->status, s);
-            if (rc == PDB_OK) {
-                cudaMemsetAsync(has_long, 0, (size_t)n_batches, s);
-                if (nnz > BSP_LONG) {
-                    k_bsp_long<<<grid_1d(nnz), 256, 0, s>>>(skey, bcol, nnz, has_long, cm->status);
-                    note_launch();
-                }
-            }
-            if (rc == PDB_OK) {
-                const void *kern = (const void *)k_bsp;
-                int grid = persistent_grid(kern, opts);
-                int32_t n32 = (int32_t)N;
-                int lossi = (int)loss;
-                uint64_t tmo = timeout_ns(opts);
-                const int64_t *rp = X->row_ptr;
-                const int32_t *cl = X->col;
-                const float *vl = X->val;
-                void *args[] = {&n32,  &batch, (void *)&n_batches, (void *)&rp, (void *)&cl, (void *)&vl,
-                                (void *)&y, &bptr, &bcol, &brow, &bval, &has_long, &cbuf, &prod, &w, &lossi, &eta, &n_epochs, &bar,
-                                (void *)&cm->status, &tmo};
-                if (cudaLaunchCooperativeKernel(kern, grid, THREADS, args, 0, s) != cudaSuccess) rc = PDB_ECUDA; note_launch();
-            }
-        }
-        for (void *p : {(void *)key, (void *)skey, (void *)tkey, (void *)bpos, (void *)tval, (void *)bcol, (void *)brow,
-                        (void *)bval, (void *)cbuf, (void *)prod, (void *)has_long, (void *)bptr, (void *)bar})
+        for (void *p : {(void *)bcol, (void *)brow, (void *)bval, (void *)cbuf, (void *)bptr, (void *)runs,
+                        (void *)n_runs})
             release(p, s);
     }
     cudaEventRecord(cm->ev_bsp1, s);
@@ -841,35 +1013,13 @@ int pdb_bsp_plan_build(const pdb_conflicts *c, int64_t batch, pdb_bsp_plan **out
         p->ev_use = nullptr;
     }
     p->n_batches = N > 0 ? (N + batch - 1) / batch : 0;
-    uint32_t *key = nullptr, *skey = nullptr, *tkey = nullptr;
-    int32_t *bpos = nullptr, *tval = nullptr;
     int rc = alloc((void **)&p->bptr, sizeof(int64_t) * (p->n_batches + 1), s);
-    if (rc == PDB_OK && nnz > 0) {
-        rc = alloc((void **)&p->bcol, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&p->brow, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&p->bval, sizeof(float) * nnz, s);
-        rc = rc ? rc : alloc((void **)&key, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&skey, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&tkey, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&bpos, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&tval, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : ensure_row_of(cm, s);
-        if (rc == PDB_OK) {
-            k_bsp_keys<<<grid_1d(nnz), 256, 0, s>>>(c->csc_pos, c->row_of, nnz, batch, key, cm->status);
-            note_launch();
-            // stable by batch: inside a batch the feature-major CSC order survives
-            rc = radix_sort(key, c->csc_pos, skey, bpos, tkey, tval, nnz, bits_for(p->n_batches - 1), cm->status, s);
-        }
-        if (rc == PDB_OK) {
-            k_bsp_gather<<<grid_1d(nnz), 256, 0, s>>>(bpos, c->col, c->val, c->row_of, nnz, p->bcol, p->brow, p->bval,
-                                                      cm->status);
-            note_launch();
-            rc = segment_bounds(skey, nnz, p->n_batches, nullptr, p->bptr, cm->status, s);
-        }
-    } else if (rc == PDB_OK) {
-        rc = fill_words(p->bptr, 0u, sizeof(int64_t) * (p->n_batches + 1), s);
-    }
-    for (void *q : {(void *)key, (void *)skey, (void *)tkey, (void *)bpos, (void *)tval}) release(q, s);
+    rc = rc ? rc : alloc((void **)&p->bcol, sizeof(int32_t) * nnz, s);
+    rc = rc ? rc : alloc((void **)&p->brow, sizeof(int32_t) * nnz, s);
+    rc = rc ? rc : alloc((void **)&p->bval, sizeof(float) * nnz, s);
+    rc = rc ? rc : alloc((void **)&p->runs, sizeof(int32_t) * nnz, s);
+    rc = rc ? rc : alloc((void **)&p->n_runs, sizeof(uint2) * std::max<int64_t>(p->n_batches, 1), s);
+    rc = rc ? rc : bsp_sort(cm, c->val, batch, p->n_batches, p->bcol, p->brow, p->bval, p->bptr, p->runs, p->n_runs, s);
     if (rc == PDB_OK && cudaPeekAtLastError() != cudaSuccess) rc = PDB_ECUDA;
     // the host keeps the batches' pair bounds (apply needs them to size its launch)
     if (rc == PDB_OK) {
@@ -906,10 +1056,8 @@ int pdb_bsp_coef(const pdb_bsp_plan *p, const pdb_csr *X, const float *y, const 
     if (row_end > row_begin && row_begin / p->batch != (row_end - 1) / p->batch) return PDB_EINVAL;
     if (row_end == row_begin) return PDB_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    k_bsp_coef<<<grid_1d((row_end - row_begin) * 32), 256, 0, s>>>(row_begin, row_end, X->row_ptr, X->col, X->val, y,
-                                                                  w, (int)loss, eta, coef, p->c->status);
-    note_launch();
-    return cudaPeekAtLastError() == cudaSuccess ? PDB_OK : PDB_ECUDA;
+    rc = launch_coef(row_begin, row_end, X, y, w, (int)loss, eta, coef, p->c->status, false, s);
+    return rc == PDB_OK && cudaPeekAtLastError() == cudaSuccess ? PDB_OK : PDB_ECUDA;
 }
 
 int pdb_bsp_apply(const pdb_bsp_plan *p, float *w, int64_t batch_index, const float *coef, void *stream)
@@ -923,12 +1071,10 @@ int pdb_bsp_apply(const pdb_bsp_plan *p, float *w, int64_t batch_index, const fl
     if (!coef) return PDB_EINVAL;
     const int64_t r0 = batch_index * p->batch, rows = std::min(p->c->n_rows, r0 + p->batch) - r0;
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((s1 - s0 + 255) / 256, (int64_t)152 * 16));
-    k_bsp_apply<<<(unsigned)blocks, 256, 0, s>>>(s0, s1, r0, rows, p->bcol, p->brow, p->bval, coef, w,
-                                                 const_cast<pdb_conflicts *>(p->c)->status);
-    note_launch();
+    const int rc = launch_apply(batch_index, r0, rows, s1 - s0, launch_info().sms, p->bptr, p->bcol, p->brow, p->bval,
+                                p->runs, p->n_runs, coef, w, const_cast<pdb_conflicts *>(p->c)->status, false, s);
     if (p->ev_use) cudaEventRecord(p->ev_use, s);
-    return cudaPeekAtLastError() == cudaSuccess ? PDB_OK : PDB_ECUDA;
+    return rc == PDB_OK && cudaPeekAtLastError() == cudaSuccess ? PDB_OK : PDB_ECUDA;
 }
 
 void pdb_bsp_plan_free(pdb_bsp_plan *p)
@@ -940,7 +1086,7 @@ void pdb_bsp_plan_free(pdb_bsp_plan *p)
         cudaEventDestroy(p->ev_use);
     }
     cudaGetLastError();
-    for (void *q : {(void *)p->bptr, (void *)p->bcol, (void *)p->brow, (void *)p->bval})
+    for (void *q : {(void *)p->bptr, (void *)p->bcol, (void *)p->brow, (void *)p->bval, (void *)p->runs, (void *)p->n_runs})
         if (q) cudaFreeAsync(q, own_stream());
     delete[] p->h_bptr;
     delete p;

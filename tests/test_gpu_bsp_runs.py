@@ -1,0 +1,72 @@
+"""BSP's run sums at the edges of their forms: runs of one to seventeen terms
+(the longest a thread sums, the shortest a block does), around the stages a
+block adds (768 terms) and their multiples, long and short runs of one feature
+set in one batch, batches of one row and of all rows, batches without a
+nonzero, rows around a warp's load (32, 256 ids).  Bit for bit the oracle's
+BSP, and so is the split form on the same data."""
+import numpy as np
+import pytest
+
+import oracle
+import synthdata
+
+torch = pytest.importorskip("torch")
+pdb = pytest.importorskip("paper_1508_00703_gb300")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    pdb.load()
+
+
+def _equal(p, batch, epochs=2):
+    p.epochs = epochs
+    X = pdb.Csr.from_problem(p)
+    y = torch.from_numpy(p.y).cuda()
+    c = pdb.pdb_build_conflicts(X)
+    ref = oracle.bsp(p, batch).view(np.uint32)
+    w = torch.zeros(p.n_cols, dtype=torch.float32, device="cuda")
+    pdb.pdb_bsp_epoch(X, y, c, w, p.loss, p.eta, batch, epochs)
+    pdb.check_status(c)
+    assert np.array_equal(w.cpu().numpy().view(np.uint32), ref)
+    w.zero_()
+    pdb.bsp_epoch_data_parallel(X, y, c, w, p.loss, p.eta, batch, epochs)
+    pdb.check_status(c)
+    assert np.array_equal(w.cpu().numpy().view(np.uint32), ref)
+
+
+def _head(n, k=6, cols=400, seed=0):
+    """Feature 0 in every row (one run of the batch's length), k - 1 others at random."""
+    rng = np.random.default_rng(seed + n)
+    col = np.stack([np.sort(np.r_[0, 1 + rng.permutation(cols - 1)[:k - 1]]) for _ in range(n)]).astype(np.int32)
+    return synthdata.from_arrays(np.arange(n + 1) * k, col.ravel(), rng.standard_normal(n * k).astype(np.float32),
+                                 np.where(rng.random(n) < 0.5, -1.0, 1.0), n_cols=cols, eta=0.01)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 6, 7, 15, 16, 17, 18, 32, 33, 191, 192, 193, 767, 768, 769, 1535, 1536, 1537, 2400])
+def test_run_lengths(n):
+    _equal(_head(n), n)
+
+
+@pytest.mark.parametrize("batch", [1, 2, 16, 17, 100, 768, 769, 5000])
+def test_batches(batch):
+    _equal(_head(1700), batch, epochs=1)
+
+
+@pytest.mark.parametrize("k", [1, 31, 32, 33, 255, 256, 257, 600])
+def test_row_lengths(k):
+    _equal(synthdata.generate("tiny", n_rows=150, n_cols=700, k=k, seed=k), 64)
+
+
+def test_batches_without_nonzeros():
+    n, empty = 90, np.arange(90) % 30 >= 10        # rows 10..29 of every 30 are empty
+    lens = np.where(empty, 0, 3)
+    rng = np.random.default_rng(5)
+    col = np.concatenate([np.sort(rng.permutation(9)[:3]) for _ in range(int((~empty).sum()))])
+    p = synthdata.from_arrays(np.r_[0, np.cumsum(lens)], col, rng.standard_normal(col.size), np.ones(n), n_cols=9)
+    for batch in (1, 10, 30, 90):
+        _equal(p, batch)
