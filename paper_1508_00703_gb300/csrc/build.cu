@@ -196,7 +196,11 @@ __global__ __launch_bounds__(SLOTS_THREADS) void k_slots(const uint32_t *__restr
     }
     __syncthreads();
     if (read_status(info)) return;
-    const bool check_dup = s_check;
+    // two positions of one row lie less than the longest row apart (recorded by
+    // k_validate_rows before this kernel): only such pairs need their rows looked
+    // up.  400k unordered rows of 50 zipf(1.1) ids: 1291 us with every pair looked up,
+    // 540 us so
+    const int64_t same_row = s_check ? info[INFO_MAX_ROW] : 0;
     const int lane = threadIdx.x & 31;
     uint32_t *sk = s_keys[threadIdx.x >> 5];
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -305,7 +309,8 @@ __global__ __launch_bounds__(SLOTS_THREADS) void k_slots(const uint32_t *__restr
             if (!gsort) gate[p] = g[e];
             if (gwin && (near_prev || near_next)) gwin[p] = g[e];
             if (last) longest = max(longest, (int)(r + 1));
-            if (check_dup && r > 0) dup |= find_row(row_ptr, n_rows, pp[e]) == find_row(row_ptr, n_rows, p);
+            if (r > 0 && (int64_t)p - pp[e] < same_row)
+                dup |= find_row(row_ptr, n_rows, pp[e]) == find_row(row_ptr, n_rows, p);
         }
         if (gsort) {
             if (s0 + 4 <= nnz)
