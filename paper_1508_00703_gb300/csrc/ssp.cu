@@ -80,16 +80,28 @@ __device__ __forceinline__ bool keep_waiting(unsigned &spins, uint64_t t0, int *
     return true;
 }
 
-// waits until counter >= need (need <= 0: at once)
+// waits until counter >= need (need <= 0: at once).  A hot feature's counter is
+// polled by thousands of lanes and every poll delays the reductions to the same
+// word, so a lane sleeps for the counts it still lacks, WAIT_NS each (about
+// what a counted access to one word costs here), instead of backing off blindly.
+// Measured, 200k examples of 20 zipf(1.0) ids, delay 1024: doubling naps of up
+// to 512 ns 4.0-6.2 ms over boxes, 4 ns per missing count 3.0, 8 ns 2.2, 12 ns
+// 1.6; the results differ by what two runs of one form differ by (which
+// examples are in flight is the same; fewer warps would be faster still, down to
+// 0.9 ms, with reads less stale).
+constexpr long long WAIT_NS = 12;
 __device__ __forceinline__ bool wait_count(const unsigned *counter, long long need, int *status, uint64_t timeout)
 {
-    if (need <= 0 || (long long)ld_acquire_u32(counter) >= need) return true;
+    if (need <= 0) return true;
+    long long have = ld_acquire_u32(counter);
+    if (have >= need) return true;
     const uint64_t t0 = globaltimer();
-    unsigned spins = 0, nap = 32;
+    unsigned spins = 0;
     for (;;) {
-        __nanosleep(nap);
-        nap = nap < 512 ? 2 * nap : 512;
-        if ((long long)ld_acquire_u32(counter) >= need) return true;
+        const long long nap = (need - have) * WAIT_NS;
+        __nanosleep(nap < 32 ? 32u : nap > 8192 ? 8192u : (unsigned)nap);
+        have = ld_acquire_u32(counter);
+        if (have >= need) return true;
         if (!keep_waiting(spins, t0, status, timeout)) return false;
     }
 }
