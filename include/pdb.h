@@ -108,7 +108,7 @@ typedef enum { PDB_LOSS_LOGISTIC = 0, PDB_LOSS_SQUARED = 1, PDB_LOSS_HINGE = 2 }
  *           publishes r + 1 with its write (the read protocol of Section 5
  *           with the iteration number counted per feature); no barrier at
  *           all.  The number lives in the same 64-bit word as the weight,
- *           with an epoch stamp: all epochs run in one pipelined launch,
+ *           counted on from epoch to epoch: all epochs run in one pipelined launch,
  *           each feature's next-epoch occurrences starting as soon as its
  *           last occurrence of the epoch has written.
  *   CHAIN   for conflict graphs that are close to one chain (a feature in
@@ -155,8 +155,9 @@ typedef enum {
 /* Launch and wait options; a zeroed struct (or NULL) selects the defaults. */
 typedef struct {
     int32_t blocks_per_sm;     /* persistent grid = blocks_per_sm x #SM (at most the occupancy
-                                  maximum); 0 = that maximum, for WINDOW 3 */
-    int32_t ticket_chunk;      /* READY: consecutive examples a warp takes per ticket; 0 = 2 */
+                                  maximum); 0 = that maximum, for WINDOW 3, for READY 2 or 4 */
+    int32_t ticket_chunk;      /* READY: consecutive examples a warp takes per ticket; 0 = 1 or 2 by
+                                  how often examples conflict, under pdb_ssp_epoch 2 */
     double wait_timeout_s;     /* limit of every device-side wait; 0 = 2 seconds; at most 10^6 seconds */
     uint64_t *trace;           /* optional (NULL = off), pdb_sgd_epoch and pdb_ssp_epoch: device array of
                                 * n_epochs * n_rows * 2 words; per example (epoch-major) the %globaltimer
@@ -262,8 +263,8 @@ int pdb_schedule_levels(const pdb_schedule *s, const int32_t **level, const int3
  * bit 31 on the last occurrence of its feature (under WINDOW with more than
  * 2^22 positions: the WINDOW engine's copy, which holds only the words of
  * positions with a near pair and 0 elsewhere); and, READY only,
- * records[n_cols] (weight bits | version << 32, the version being the rank
- * waited for in bits 0..28 and an epoch stamp 1..7 in bits 29..31;
+ * records[n_cols] (weight bits | version << 32; in epoch e the occurrence of
+ * rank r waits for version e * n_rows + r, modulo 2^32;
  * meaningful while pdb_sgd_epoch runs; NULL under WINDOW).  PDB_ESTATE for LEVELS and CHAIN
  * schedules. */
 int pdb_schedule_ready(const pdb_schedule *s, const uint32_t **gate, const uint64_t **records);

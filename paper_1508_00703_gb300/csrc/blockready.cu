@@ -41,28 +41,19 @@ constexpr int BR_WARPS = 32;           // most warps
 
 // warp_combine inside groups of LPE lanes (rows of at most LPE ids, or 32 lanes):
 // the partials of the lanes that a group does not have are +0, added once (a
-// second addition of +0 changes nothing); the rest of the tree in rounds of
-// independent shuffles with the operands of the one-level-per-shuffle form.
+// second addition of +0 changes nothing).
 template <int LPE>
 __device__ __forceinline__ float combine_group(float a)
 {
+    if (LPE == 32) return warp_combine_latency(a);
+    const float z = __fadd_rn(a, 0.0f);
     float n;
-    if (LPE == 32) {
-        const float b16 = __shfl_xor_sync(FULL, a, 16), b8 = __shfl_xor_sync(FULL, a, 8);
-        const float b24 = __shfl_xor_sync(FULL, a, 24), b4 = __shfl_xor_sync(FULL, a, 4);
-        const float b20 = __shfl_xor_sync(FULL, a, 20), b12 = __shfl_xor_sync(FULL, a, 12);
-        const float b28 = __shfl_xor_sync(FULL, a, 28);
-        n = __fadd_rn(__fadd_rn(__fadd_rn(a, b16), __fadd_rn(b8, b24)),
-                      __fadd_rn(__fadd_rn(b4, b20), __fadd_rn(b12, b28)));
+    if (LPE == 16) {
+        const float b8 = __shfl_xor_sync(FULL, z, 8), b4 = __shfl_xor_sync(FULL, z, 4);
+        const float b12 = __shfl_xor_sync(FULL, z, 12);
+        n = __fadd_rn(__fadd_rn(z, b8), __fadd_rn(b4, b12));
     } else {
-        const float z = __fadd_rn(a, 0.0f);
-        if (LPE == 16) {
-            const float b8 = __shfl_xor_sync(FULL, z, 8), b4 = __shfl_xor_sync(FULL, z, 4);
-            const float b12 = __shfl_xor_sync(FULL, z, 12);
-            n = __fadd_rn(__fadd_rn(z, b8), __fadd_rn(b4, b12));
-        } else {
-            n = __fadd_rn(z, __shfl_xor_sync(FULL, z, 4));
-        }
+        n = __fadd_rn(z, __shfl_xor_sync(FULL, z, 4));
     }
     const float c2 = __shfl_xor_sync(FULL, n, 2), c1 = __shfl_xor_sync(FULL, n, 1), c3 = __shfl_xor_sync(FULL, n, 3);
     return __fadd_rn(__fadd_rn(n, c2), __fadd_rn(c1, c3));

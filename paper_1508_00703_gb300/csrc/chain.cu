@@ -223,21 +223,6 @@ __device__ __forceinline__ float combine4(float a0, float a1, float a2, float a3
                      __fadd_rn(__fadd_rn(b1, b5), __fadd_rn(b3, b7)));
 }
 
-// One partial per lane: the whole tree in two rounds of independent shuffles.
-// The first brings the leaves of lanes l ^ 16, 8, 24, 4, 20, 12, 28 and adds
-// levels 16, 8 and 4 locally, the second the results of lanes l ^ 2, 1, 3.
-__device__ __forceinline__ float combine1(float a)
-{
-    const float b16 = __shfl_xor_sync(FULL, a, 16), b8 = __shfl_xor_sync(FULL, a, 8);
-    const float b24 = __shfl_xor_sync(FULL, a, 24), b4 = __shfl_xor_sync(FULL, a, 4);
-    const float b20 = __shfl_xor_sync(FULL, a, 20), b12 = __shfl_xor_sync(FULL, a, 12);
-    const float b28 = __shfl_xor_sync(FULL, a, 28);
-    const float n = __fadd_rn(__fadd_rn(__fadd_rn(a, b16), __fadd_rn(b8, b24)),
-                              __fadd_rn(__fadd_rn(b4, b20), __fadd_rn(b12, b28)));
-    const float c2 = __shfl_xor_sync(FULL, n, 2), c1 = __shfl_xor_sync(FULL, n, 1), c3 = __shfl_xor_sync(FULL, n, 3);
-    return __fadd_rn(__fadd_rn(n, c2), __fadd_rn(c1, c3));
-}
-
 // What the compute warp carries from example to example.
 template <int R>
 struct ChainWarp {
@@ -306,7 +291,7 @@ __device__ __forceinline__ void chain_example(ChainWarp<R> &cw, int wslot, int x
 #pragma unroll
         for (int q = 0; q < R; ++q) a = __fmaf_rn(w[q], cw.x[q], a);
         if (TRACE) trace_mark(trace, idx, 0);    // every weight is read
-        m = combine1(a);
+        m = warp_combine_latency(a);
     }
     const float c = FAST ? dev_step_fast(LOSS, m, y, eta, cw.redo) : __fmul_rn(eta, dev_grad(LOSS, m, y));
     if (TRACE) trace_mark(trace, idx, 1);    // before any write is visible

@@ -274,6 +274,15 @@ __device__ __forceinline__ float dev_step_fast(int loss, float m, float y, float
     return __fmul_rn(eta, dev_grad(loss, m, y));
 }
 
+// dev_step_fast, with the general form where it must be taken
+__device__ __forceinline__ float dev_step(int loss, float m, float y, float eta)
+{
+    bool redo = false;
+    float c = dev_step_fast(loss, m, y, eta, redo);
+    if (redo) c = __fmul_rn(eta, dev_grad(loss, m, y));
+    return c;
+}
+
 // combine the 32 lane partial sums pairwise: xor 16, 8, 4, 2, 1 (every lane
 // ends with the same value because fp32 addition commutes)
 __device__ __forceinline__ float warp_combine(float a)
@@ -281,6 +290,23 @@ __device__ __forceinline__ float warp_combine(float a)
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) a = __fadd_rn(a, __shfl_xor_sync(FULL, a, off));
     return a;
+}
+
+// The same in two rounds of independent shuffles (~85 cycles against ~145, but
+// ten shuffles for five: for engines bound by one example's latency): the first
+// brings the leaves of lanes l ^ 16, 8, 24, 4, 20, 12, 28 and adds the levels 16,
+// 8 and 4 locally, the second the results of lanes l ^ 2, 1, 3.  Every addition
+// has the operands that the one-level-per-shuffle form gives it, so the same bits.
+__device__ __forceinline__ float warp_combine_latency(float a)
+{
+    const float b16 = __shfl_xor_sync(FULL, a, 16), b8 = __shfl_xor_sync(FULL, a, 8);
+    const float b24 = __shfl_xor_sync(FULL, a, 24), b4 = __shfl_xor_sync(FULL, a, 4);
+    const float b20 = __shfl_xor_sync(FULL, a, 20), b12 = __shfl_xor_sync(FULL, a, 12);
+    const float b28 = __shfl_xor_sync(FULL, a, 28);
+    const float n = __fadd_rn(__fadd_rn(__fadd_rn(a, b16), __fadd_rn(b8, b24)),
+                              __fadd_rn(__fadd_rn(b4, b20), __fadd_rn(b12, b28)));
+    const float c2 = __shfl_xor_sync(FULL, n, 2), c1 = __shfl_xor_sync(FULL, n, 1), c3 = __shfl_xor_sync(FULL, n, 3);
+    return __fadd_rn(__fadd_rn(n, c2), __fadd_rn(c1, c3));
 }
 
 // Gate word of a position (the conflicts' per-position schedule input):

@@ -45,20 +45,6 @@ struct DenseSmem {
     float y[DN_RING * DN_G];
 };
 
-// the tree of warp_combine in two rounds of independent shuffles (the
-// additions and their operands are the same)
-__device__ __forceinline__ float combine_two_rounds(float a)
-{
-    const float b16 = __shfl_xor_sync(FULL, a, 16), b8 = __shfl_xor_sync(FULL, a, 8);
-    const float b24 = __shfl_xor_sync(FULL, a, 24), b4 = __shfl_xor_sync(FULL, a, 4);
-    const float b20 = __shfl_xor_sync(FULL, a, 20), b12 = __shfl_xor_sync(FULL, a, 12);
-    const float b28 = __shfl_xor_sync(FULL, a, 28);
-    const float n = __fadd_rn(__fadd_rn(__fadd_rn(a, b16), __fadd_rn(b8, b24)),
-                              __fadd_rn(__fadd_rn(b4, b20), __fadd_rn(b12, b28)));
-    const float c2 = __shfl_xor_sync(FULL, n, 2), c1 = __shfl_xor_sync(FULL, n, 1), c3 = __shfl_xor_sync(FULL, n, 3);
-    return __fadd_rn(__fadd_rn(n, c2), __fadd_rn(c1, c3));
-}
-
 template <int R>
 __device__ __forceinline__ void load_values(const DenseSmem<R> &S, int slot, int lane, float (&x)[R])
 {
@@ -106,7 +92,7 @@ __device__ __forceinline__ float dense_example(const DenseSmem<R> &S, float (&w)
         xp[q + 3] = v.w;
     }
     if (TRACE) trace_mark(trace, idx, 0);
-    const float m = combine_two_rounds(a);
+    const float m = warp_combine_latency(a);
     bool general = false;
     float s = dev_step_fast(LOSS, m, y, eta, general);
     if (LOSS == PDB_LOSS_LOGISTIC && general) s = __fmul_rn(eta, dev_grad(LOSS, m, y));

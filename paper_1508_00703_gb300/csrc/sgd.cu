@@ -118,14 +118,13 @@ __global__ __launch_bounds__(THREADS) void k_sgd_levels(int32_t n_rows, const in
 // together with version r + 1 in one 64-bit store (Write Constraint: its own
 // read, the only read of that version, came first).  Both halves travel in
 // one single-copy-atomic access, so no fence is needed.
-// All epochs run in one launch, pipelined: a version carries the epoch's
-// stamp (1..7, bits 29-31 above the 29-bit rank), and the last occurrence
-// of j in an epoch (GATE_LAST) publishes version 0 with the next epoch's
-// stamp, so the next epoch's first occurrence of j starts as soon as that
-// write lands -- not at a kernel boundary (exact by Theorem 2: per feature
-// the order is still the data order, epoch after epoch).  A record only
-// ever holds a version of the current or the previous epoch of its
-// feature, so stamps that repeat every 7 epochs never match stale ones.
+// All epochs run in one launch, pipelined: rank r of epoch e waits for version
+// e * n_rows + r (a rank is below n_rows), and the last occurrence of j in an
+// epoch (GATE_LAST) publishes (e + 1) * n_rows, so the next epoch's first
+// occurrence of j starts as soon as that write lands -- not at a kernel
+// boundary (exact by Theorem 2: per feature the order is still the data order,
+// epoch after epoch).  Versions count modulo 2^32: two that are equal lie
+// 2^31 examples or more apart, far more than are ever in flight.
 // Examples are taken in data order (epoch-major) from a ticket counter,
 // `chunk` consecutive ones at a time and run in order by the warp that took
 // them, so the oldest unfinished example never waits on a younger one and
@@ -142,55 +141,43 @@ __device__ __forceinline__ void st_rec(unsigned long long *p, float w, unsigned 
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Gathers w for the lane's elements, waiting until each record carries the
-// wanted version.  False when the wait gave up (timeout or a failure
-// elsewhere recorded in status).
+// Gathers w for the lane's elements (bit r of `pending`: the lane has element r),
+// waiting until each record carries the wanted version; called by the whole
+// warp.  False when the wait gave up (timeout or a failure elsewhere recorded in
+// status).  The loop is the warp's, not each lane's: lanes that left it one by
+// one would stay apart, and every shuffle after it would first have to bring
+// them together again (~280 cycles each, measured).
 template <int R>
 __device__ __forceinline__ bool gather_ready(const unsigned long long *rec, const int *j, const unsigned *want,
-                                             float *wv, int lane, int k, int *status, uint64_t timeout)
+                                             unsigned pending, float *wv, int *status, uint64_t timeout)
 {
-    unsigned pending = 0;
+    uint64_t t0 = 0;
+    for (unsigned spins = 0;; ++spins) {
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (r * 32 + lane < k) {
-            unsigned long long v = ld_rec(rec + j[r]);
-            wv[r] = __uint_as_float((unsigned)v);
-            if ((unsigned)(v >> 32) != want[r]) pending |= 1u << r;
+        for (int r = 0; r < R; ++r) {
+            unsigned long long v = 0;
+            if (pending & (1u << r)) v = ld_rec(rec + j[r]);
+            const bool hit = (pending & (1u << r)) && (unsigned)(v >> 32) == want[r];
+            wv[r] = hit ? __uint_as_float((unsigned)v) : wv[r];
+            pending &= hit ? ~(1u << r) : ~0u;
         }
-    if (pending == 0) return true;
-    const uint64_t t0 = globaltimer();
-    unsigned spins = 0, nap = 32;
-    while (pending) {
-        // back off so a waiting lane does not flood L2 with polls; the cap
-        // (128 ns) is the latency of a hop on mid-conflict data, where READY
-        // is AUTO's choice (512 ns was 16% slower on the tiny workload)
-        __nanosleep(nap);
-        nap = nap < 128 ? 2 * nap : 128;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (pending & (1u << r)) {
-                unsigned long long v = ld_rec(rec + j[r]);
-                if ((unsigned)(v >> 32) == want[r]) {
-                    wv[r] = __uint_as_float((unsigned)v);
-                    pending &= ~(1u << r);
-                }
-            }
-        if (pending && (++spins & 15u) == 0) {
-            if (read_status(status)) return false;
-            if (globaltimer() - t0 > timeout) {
+        if (!__any_sync(FULL, pending)) return true;
+        if ((spins & 31u) == 31u) {
+            const uint64_t now = globaltimer();
+            if (spins == 31u) t0 = now;
+            bool stop = read_status(status) != 0;
+            if (!stop && now - t0 > timeout) {
                 set_status(status, PDB_ETIMEOUT);
-                return false;
+                stop = true;
             }
+            if (__any_sync(FULL, stop)) return false;
         }
     }
-    return true;
 }
 
 // one example under the ready protocol; false when a wait gave up
-__host__ __device__ __forceinline__ unsigned epoch_stamp(int64_t e) { return (1u + (unsigned)(e % 7)) << 29; }
-
 template <int R>
-__device__ __forceinline__ bool ready_example(int t, unsigned stamp, unsigned next_stamp,
+__device__ __forceinline__ bool ready_example(int t, unsigned base, unsigned next_base,
                                               const int64_t *__restrict__ row_ptr,
                                               const int32_t *__restrict__ col, const float *__restrict__ val,
                                               const float *__restrict__ y, const uint32_t *__restrict__ gate,
@@ -204,26 +191,26 @@ __device__ __forceinline__ bool ready_example(int t, unsigned stamp, unsigned ne
     if (k <= 32 * R) {
         int j[R];
         float x[R], wv[R];
-        unsigned want[R], next[R];
+        unsigned want[R], next[R], have = 0;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             int i = r * 32 + lane;
+            have |= i < k ? 1u << r : 0u;
             j[r] = i < k ? col[b + i] : 0;
             x[r] = i < k ? (val ? val[b + i] : 1.0f) : 0.0f;
             uint32_t g = i < k ? gate[b + i] : 0u;
-            want[r] = (g & GATE_RANK) | stamp;
-            next[r] = (g & GATE_LAST) ? next_stamp : want[r] + 1u;
+            want[r] = base + (g & GATE_RANK);
+            next[r] = (g & GATE_LAST) ? next_base : want[r] + 1u;
             wv[r] = 0.0f;
         }
-        bool ok = gather_ready<R>(rec, j, want, wv, lane, k, status, timeout);
-        if (!__all_sync(FULL, ok)) return false;
+        if (!gather_ready<R>(rec, j, want, have, wv, status, timeout)) return false;
         trace_mark(trace, idx, 0);
         float acc = 0.0f;
 #pragma unroll
         for (int r = 0; r < R; ++r)
             if (r * 32 + lane < k) acc = __fmaf_rn(wv[r], x[r], acc);
-        const float m = warp_combine(acc);
-        const float c = __fmul_rn(eta, dev_grad(loss, m, yt));
+        const float m = warp_combine_latency(acc);
+        const float c = dev_step(loss, m, yt, eta);
         trace_mark(trace, idx, 1);   // before any write is visible
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -234,25 +221,24 @@ __device__ __forceinline__ bool ready_example(int t, unsigned stamp, unsigned ne
     // (this example owns its features until it writes them, so re-reading
     // the records returns the same weights)
     float acc = 0.0f;
-    bool ok = true;
-    for (int i = lane; i < k && ok; i += 32) {
-        int j1[1] = {col[b + i]};
-        unsigned w1[1] = {(gate[b + i] & GATE_RANK) | stamp};
-        float v1[1];
-        ok = gather_ready<1>(rec, j1, w1, v1, 0, 1, status, timeout);
-        if (ok) acc = __fmaf_rn(v1[0], val ? val[b + i] : 1.0f, acc);
+    for (int i = lane; i - lane < k; i += 32) {
+        const bool in = i < k;
+        const int j1[1] = {in ? col[b + i] : 0};
+        const unsigned w1[1] = {in ? base + (gate[b + i] & GATE_RANK) : 0u};
+        float v1[1] = {0.0f};
+        if (!gather_ready<1>(rec, j1, w1, in ? 1u : 0u, v1, status, timeout)) return false;
+        if (in) acc = __fmaf_rn(v1[0], val ? val[b + i] : 1.0f, acc);
     }
-    if (!__all_sync(FULL, ok)) return false;
     trace_mark(trace, idx, 0);
-    const float m = warp_combine(acc);
-    const float c = __fmul_rn(eta, dev_grad(loss, m, yt));
+    const float m = warp_combine_latency(acc);
+    const float c = dev_step(loss, m, yt, eta);
     trace_mark(trace, idx, 1);   // before any write is visible
     for (int i = lane; i < k; i += 32) {
         const int jj = col[b + i];
         const float xx = val ? val[b + i] : 1.0f;
         const uint32_t g = gate[b + i];
         const float wo = __uint_as_float((unsigned)ld_rec(rec + jj));
-        st_rec(rec + jj, __fsub_rn(wo, __fmul_rn(c, xx)), (g & GATE_LAST) ? next_stamp : ((g & GATE_RANK) + 1u) | stamp);
+        st_rec(rec + jj, __fsub_rn(wo, __fmul_rn(c, xx)), (g & GATE_LAST) ? next_base : base + (g & GATE_RANK) + 1u);
     }
     return true;
 }
@@ -276,8 +262,9 @@ __global__ __launch_bounds__(THREADS) void k_sgd_ready(int32_t n_rows, const int
         const int64_t t1 = min64(total, (int64_t)tk + chunk);
         for (int64_t tg = (int64_t)tk; tg < t1; ++tg) {
             const int64_t e = tg / n_rows;
-            if (!ready_example<R>((int)(tg - e * n_rows), epoch_stamp(e), epoch_stamp(e + 1), row_ptr, col, val, y,
-                                  gate, rec, loss, eta, status, timeout, trace, tg))
+            const unsigned base = (unsigned)e * (unsigned)n_rows;
+            if (!ready_example<R>((int)(tg - e * n_rows), base, base + (unsigned)n_rows, row_ptr, col, val, y, gate, rec,
+                                  loss, eta, status, timeout, trace, tg))
                 return;
         }
     }
@@ -288,9 +275,8 @@ __global__ __launch_bounds__(THREADS) void k_sgd_ready(int32_t n_rows, const int
 __global__ void k_pack(const float *__restrict__ w, int64_t n, unsigned long long *__restrict__ rec, const int *status)
 {
     if (read_status(status)) return;
-    const unsigned long long v0 = (unsigned long long)epoch_stamp(0) << 32;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        rec[i] = (unsigned long long)__float_as_uint(w[i]) | v0;
+        rec[i] = (unsigned long long)__float_as_uint(w[i]);
 }
 
 __global__ void k_unpack(const unsigned long long *__restrict__ rec, int64_t n, float *__restrict__ w,
@@ -791,6 +777,26 @@ int launch_apply(int64_t bi, int64_t r0, int64_t rows, int64_t pairs, int sms, c
     return e == cudaSuccess ? PDB_OK : PDB_ECUDA;
 }
 
+// The grid of k_sgd_ready and the examples a warp takes per ticket.  Two
+// examples of k ids conflict with probability ~k^2 / n_cols, so about n_cols /
+// k^2 run at once.  Where those are few, a warp's second example per ticket, which
+// waits for the first and is loaded only after it, lengthens every chain, and
+// warps beyond them only poll; where they are many, the warps cover memory
+// latency, and the tickets (one address) bound short rows.  Measured, ms per epoch, 1
+// example per ticket with 2 blocks per SM / 2 with 4: 200k examples of 30 ids over 200k
+// features (n_cols / k^2 = 222) 1.39 / 3.29; 100k of 60 over 4M (1111) 0.16 / 0.50;
+// 500k of 100 over 100M (10000) 2.06 / 2.25 (2.32 at full occupancy); 500k of 30
+// over 20M (22222) 0.59 / 0.38.
+int ready_grid(const void *kern, const pdb_csr *X, const pdb_opts *opts, int *chunk)
+{
+    const double k = X->n_rows > 0 ? (double)X->nnz / (double)X->n_rows : 0.0;
+    const bool free = (double)X->n_cols > 5000.0 * k * k;
+    *chunk = opts && opts->ticket_chunk > 0 ? opts->ticket_chunk : free ? 2 : 1;
+    pdb_opts o = opts ? *opts : pdb_opts{};
+    if (o.blocks_per_sm <= 0) o.blocks_per_sm = free ? 4 : 2;
+    return persistent_grid(kern, &o);
+}
+
 int check_run(const pdb_csr *X, const float *y, const pdb_conflicts *c, const float *w, int loss, int epochs)
 {
     if (!X || !c || epochs < 0) return PDB_EINVAL;
@@ -858,9 +864,9 @@ int pdb_sgd_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, cons
             cudaEventRecord(cm->ev_k1, s);
         } else {
             auto kern = width == 2 ? k_sgd_ready<2> : width == 4 ? k_sgd_ready<4> : k_sgd_ready<8>;
-            int grid = persistent_grid((const void *)kern, opts);
+            int chunk = 1;
+            const int grid = ready_grid((const void *)kern, X, opts, &chunk);
             const int64_t F = X->n_cols;
-            const int chunk = (opts && opts->ticket_chunk > 0) ? opts->ticket_chunk : 2;
             k_pack<<<grid_1d(F), 256, 0, s>>>(w, F, h->rec, cm->status);
             note_launch();
             if (fill_words(h->ticket, 0u, sizeof(unsigned long long), s) != PDB_OK) return PDB_ECUDA;
@@ -1207,14 +1213,15 @@ extern "C" int pdb_sgd_epoch_ready_noalloc(const pdb_csr *X, const float *y, con
         const int64_t F = X->n_cols;
         const int32_t n32 = (int32_t)X->n_rows;
         const uint64_t tmo = timeout_ns(nullptr);
-        const int grid = persistent_grid((const void *)k_sgd_ready<8>, nullptr);
+        int chunk = 1;
+        const int grid = ready_grid((const void *)k_sgd_ready<8>, X, nullptr, &chunk);
         if (F > 0) {
             k_pack<<<grid_1d(F), 256, 0, s>>>(w, F, rec, status);
             note_launch();
         }
         if (fill_words(ticket, 0u, sizeof(unsigned long long), s) != PDB_OK) return PDB_ECUDA;
         k_sgd_ready<8><<<grid, THREADS, 0, s>>>(n32, X->row_ptr, X->col, X->val, y, gate, rec, (int)loss, eta,
-                                                n_epochs, ticket, 2, status, tmo, nullptr);
+                                                n_epochs, ticket, chunk, status, tmo, nullptr);
         note_launch();
         if (F > 0) {
             k_unpack<<<grid_1d(F), 256, 0, s>>>(rec, F, w, status);
