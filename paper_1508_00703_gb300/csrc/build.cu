@@ -100,18 +100,43 @@ __global__ void k_row_of(const int64_t *__restrict__ row_ptr, int64_t n_rows, in
     }
 }
 
-// the example holding position p: the last t with row_ptr[t] <= p
-__device__ __forceinline__ int64_t find_row(const int64_t *__restrict__ row_ptr, int64_t n_rows, int64_t p)
+// the end of the example holding position p (the t with row_ptr[t] <= p <
+// row_ptr[t + 1]), found from where rows of one length would put it: two loads
+// of neighbours there, a gallop and a binary search otherwise.  rows_per_pos =
+// n_rows / n_positions as a 32.32 fixed-point number.
+__device__ __forceinline__ int64_t row_end(const int64_t *__restrict__ row_ptr, int64_t n_rows, int64_t p,
+                                           uint64_t rows_per_pos)
 {
-    int64_t lo = 0, hi = n_rows - 1;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
+    const uint64_t est = __umul64hi((uint64_t)p << 32, rows_per_pos);      // p * n_rows / n_positions
+    const int64_t g = min((int64_t)est, n_rows - 1);
+    const int64_t a = row_ptr[g], e = row_ptr[g + 1];
+    if (a <= p && p < e) return e;
+    int64_t lo, hi, step = 1;               // row_ptr[lo] <= p < row_ptr[hi]
+    if (a > p) {
+        hi = g;
+        lo = g - 1;
+        while (lo > 0 && row_ptr[lo] > p) {
+            hi = lo;
+            step *= 2;
+            lo = max((int64_t)0, hi - step);
+        }
+    } else {
+        lo = g + 1;
+        hi = g + 2;
+        while (hi < n_rows && row_ptr[hi] <= p) {
+            lo = hi;
+            step *= 2;
+            hi = min(n_rows, lo + step);
+        }
+    }
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
         if (row_ptr[mid] <= p)
             lo = mid;
         else
-            hi = mid - 1;
+            hi = mid;
     }
-    return lo;
+    return row_ptr[lo + 1];
 }
 
 // The first slot of the run of key skey[q] (keys sorted): a gallop back from
@@ -198,9 +223,10 @@ __global__ __launch_bounds__(SLOTS_THREADS) void k_slots(const uint32_t *__restr
     if (read_status(info)) return;
     // two positions of one row lie less than the longest row apart (recorded by
     // k_validate_rows before this kernel): only such pairs need their rows looked
-    // up.  400k unordered rows of 50 zipf(1.1) ids: 1291 us with every pair looked up,
-    // 540 us so
+    // up.  400k unordered rows of 50 zipf(1.1) ids: 1291 us with both rows of every pair
+    // searched for, 540 for such pairs only, 283 with row_end
     const int64_t same_row = s_check ? info[INFO_MAX_ROW] : 0;
+    const uint64_t rows_per_pos = s_check ? ((uint64_t)n_rows << 32) / (uint64_t)nnz : 0;
     const int lane = threadIdx.x & 31;
     uint32_t *sk = s_keys[threadIdx.x >> 5];
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -309,8 +335,7 @@ __global__ __launch_bounds__(SLOTS_THREADS) void k_slots(const uint32_t *__restr
             if (!gsort) gate[p] = g[e];
             if (gwin && (near_prev || near_next)) gwin[p] = g[e];
             if (last) longest = max(longest, (int)(r + 1));
-            if (r > 0 && (int64_t)p - pp[e] < same_row)
-                dup |= find_row(row_ptr, n_rows, pp[e]) == find_row(row_ptr, n_rows, p);
+            if (r > 0 && (int64_t)p - pp[e] < same_row) dup |= p < row_end(row_ptr, n_rows, pp[e], rows_per_pos);
         }
         if (gsort) {
             if (s0 + 4 <= nnz)

@@ -40,6 +40,22 @@ def test_repeat_in_a_row(longest, row):
         assert _status(lens, np.concatenate(bad), 400) == pdb.PDB_EDUP
 
 
+@pytest.mark.parametrize("lens", ["ragged", "empty ends", "one long"])
+def test_rows_found_from_any_position(lens):
+    # rows far from where rows of one length would put them: the repeat sits in each row in turn
+    rng = np.random.default_rng(9)
+    n = 120
+    k = {"ragged": rng.integers(0, 40, n), "empty ends": np.where((np.arange(n) > 40) & (np.arange(n) < 60), 30, 0),
+         "one long": np.where(np.arange(n) == 100, 300, 2)}[lens]
+    rows = [rng.permutation(500)[:m] for m in k]
+    assert _status(k, np.concatenate(rows), 500) == pdb.PDB_OK
+    for t in np.flatnonzero(k >= 2):
+        bad = [r.copy() for r in rows]
+        a, b = np.sort(rng.choice(k[t], 2, replace=False))
+        bad[t][b] = bad[t][a]
+        assert _status(k, np.concatenate(bad), 500) == pdb.PDB_EDUP, t
+
+
 def test_same_ids_in_neighbouring_rows():
     lens = np.array([3, 1, 2, 0, 3, 1])
     assert _status(lens, np.array([5, 2, 7, 7, 5, 2, 7, 5, 2, 2]), 8) == pdb.PDB_OK
