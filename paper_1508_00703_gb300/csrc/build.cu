@@ -225,7 +225,8 @@ __global__ __launch_bounds__(SLOTS_THREADS) void k_slots(const uint32_t *__restr
     // k_validate_rows before this kernel): only such pairs need their rows looked
     // up.  400k unordered rows of 50 zipf(1.1) ids: 1291 us with both rows of every pair
     // searched for, 540 for such pairs only, 283 with row_end
-    const int64_t same_row = s_check ? info[INFO_MAX_ROW] : 0;
+    const bool check_dup = s_check;
+    const int same_row = s_check ? info[INFO_MAX_ROW] : 0;
     const uint64_t rows_per_pos = s_check ? ((uint64_t)n_rows << 32) / (uint64_t)nnz : 0;
     const int lane = threadIdx.x & 31;
     uint32_t *sk = s_keys[threadIdx.x >> 5];
@@ -335,7 +336,7 @@ __global__ __launch_bounds__(SLOTS_THREADS) void k_slots(const uint32_t *__restr
             if (!gsort) gate[p] = g[e];
             if (gwin && (near_prev || near_next)) gwin[p] = g[e];
             if (last) longest = max(longest, (int)(r + 1));
-            if (r > 0 && (int64_t)p - pp[e] < same_row) dup |= p < row_end(row_ptr, n_rows, pp[e], rows_per_pos);
+            if (check_dup && r > 0 && p - pp[e] < same_row) dup |= p < row_end(row_ptr, n_rows, pp[e], rows_per_pos);
         }
         if (gsort) {
             if (s0 + 4 <= nnz)
@@ -384,27 +385,39 @@ __global__ __launch_bounds__(SLOTS_THREADS) void k_slots(const uint32_t *__restr
 // (positions are a permutation of the slots).  One thread block inverts that
 // piece in shared memory and writes it out contiguously: no ranking, and
 // DRAM sees whole lines instead of one scattered 4-byte store per slot.
-constexpr int SCATTER_SB = 14;                 // 2^14 slots = 64 KB of shared memory per block
-constexpr int SCATTER_THREADS = 512;
-__global__ __launch_bounds__(SCATTER_THREADS) void k_scatter_block(const uint32_t *__restrict__ ppos,
+template <int SB>
+constexpr int SCATTER_THREADS = SB == 15 ? 1024 : 512;
+template <int SB>
+__global__ __launch_bounds__(SCATTER_THREADS<SB>) void k_scatter_block(const uint32_t *__restrict__ ppos,
                                                                   const uint32_t *__restrict__ pgate, int64_t nnz,
                                                                   uint32_t *__restrict__ gate, int *info)
 {
     extern __shared__ uint32_t piece[];
     if (read_status(info)) return;
-    const int64_t base = (int64_t)blockIdx.x << SCATTER_SB;
-    const int cnt = (int)min64((int64_t)1 << SCATTER_SB, nnz - base);
+    const int64_t base = (int64_t)blockIdx.x << SB;
+    const int cnt = (int)min64((int64_t)1 << SB, nnz - base);
     bool bad = false;
-    for (int i = threadIdx.x; i < cnt; i += SCATTER_THREADS) {
-        const uint32_t off = __ldcs(ppos + base + i) - (uint32_t)base;
-        if (off < (uint32_t)cnt)
-            piece[off] = __ldcs(pgate + base + i);
-        else
-            bad = true;
+    // 8 pairs per thread in flight
+    for (int i0 = threadIdx.x; i0 < cnt; i0 += 8 * SCATTER_THREADS<SB>) {
+        uint32_t off[8], g[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 + u * SCATTER_THREADS<SB>;
+            off[u] = i < cnt ? __ldcs(ppos + base + i) - (uint32_t)base : 0u;
+            g[u] = i < cnt ? __ldcs(pgate + base + i) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (i0 + u * SCATTER_THREADS<SB> >= cnt) break;
+            if (off[u] < (uint32_t)cnt)
+                piece[off[u]] = g[u];
+            else
+                bad = true;
+        }
     }
     if (bad) set_status(info, PDB_EFAULT);
     __syncthreads();
-    for (int i = threadIdx.x; i < cnt; i += SCATTER_THREADS) gate[base + i] = piece[i];
+    for (int i = threadIdx.x; i < cnt; i += SCATTER_THREADS<SB>) gate[base + i] = piece[i];
 }
 
 // Position order: rank, previous and next occurrence of each position's feature.
@@ -659,10 +672,38 @@ int ensure_row_of(pdb_conflicts *c, cudaStream_t s)
 
 namespace {
 
+// sorts the (position, gate word) pairs on the position bits above SB and
+// inverts each 2^SB-slot block of them (2^(SB + 2) bytes of shared memory)
+template <int SB>
+int scatter_gate(const pdb_conflicts *c, uint32_t *pk, int32_t *pv, uint32_t *tkey, int32_t *tval, uint32_t *gate,
+                 cudaStream_t s)
+{
+    const int64_t nnz = c->nnz;
+    const int rc = radix_sort_bits((const uint32_t *)c->csc_pos, (const int32_t *)c->gate_sorted, pk, pv, tkey, tval, nnz,
+                                   SB, bits_for(nnz - 1), c->info, s);
+    if (rc != PDB_OK) return rc;
+    const size_t smem = sizeof(uint32_t) << SB;
+    // set once per device (any device past the table: every call)
+    static std::atomic<bool> configured[64];
+    const bool known = c->device >= 0 && c->device < 64;
+    if (!known || !configured[c->device].load(std::memory_order_acquire)) {
+        if (cudaFuncSetAttribute(k_scatter_block<SB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess)
+            return PDB_ECUDA;
+        if (known) configured[c->device].store(true, std::memory_order_release);
+    }
+    const int64_t blocks = ((nnz - 1) >> SB) + 1;
+    k_scatter_block<SB><<<(unsigned)blocks, SCATTER_THREADS<SB>, smem, s>>>(pk, (const uint32_t *)pv, nnz, gate, c->info);
+    note_launch();
+    return PDB_OK;
+}
+
 // The position-order gate array (idempotent; enqueued on s).  Above 2^22
-// positions the build keeps the gate words in csc_pos order only; here the
-// (position, gate) pairs are sorted on the position bits above SCATTER_SB
-// and k_scatter_block inverts each 2^SCATTER_SB-slot block in shared memory.
+// positions the build keeps the gate words in csc_pos order only; they are
+// brought to position order here.  Blocks of 2^14 slots keep three thread blocks
+// per SM; 2^15 leave one, but for 25 position bits (inputs of 2^24 to 2^25) one
+// radix pass of 10 bits then does where 2^14 takes two.  20M positions:
+// passes and blocks 265 us with 2^14, 219 so.
 int ensure_gate(pdb_conflicts *c, cudaStream_t s)
 {
     if (c->gate) return PDB_OK;
@@ -675,27 +716,8 @@ int ensure_gate(pdb_conflicts *c, cudaStream_t s)
     rc = rc ? rc : alloc((void **)&tkey, sizeof(uint32_t) * nnz, s);
     rc = rc ? rc : alloc((void **)&tval, sizeof(int32_t) * nnz, s);
     if (rc == PDB_OK)
-        rc = radix_sort_bits((const uint32_t *)c->csc_pos, (const int32_t *)c->gate_sorted, pk, pv, tkey, tval, nnz,
-                             SCATTER_SB, bits_for(nnz - 1), c->info, s);
-    if (rc == PDB_OK) {
-        const size_t smem = sizeof(uint32_t) << SCATTER_SB;
-        // set once per device (any device past the table: every call)
-        static std::atomic<bool> configured[64];
-        const bool known = c->device >= 0 && c->device < 64;
-        if (!known || !configured[c->device].load(std::memory_order_acquire)) {
-            if (cudaFuncSetAttribute(k_scatter_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-                cudaSuccess)
-                rc = PDB_ECUDA;
-            else if (known)
-                configured[c->device].store(true, std::memory_order_release);
-        }
-        if (rc == PDB_OK) {
-            const int64_t blocks = ((nnz - 1) >> SCATTER_SB) + 1;
-            k_scatter_block<<<(unsigned)blocks, SCATTER_THREADS, smem, s>>>(pk, (const uint32_t *)pv, nnz, gate,
-                                                                             c->info);
-            note_launch();
-        }
-    }
+        rc = bits_for(nnz - 1) == 25 ? scatter_gate<15>(c, pk, pv, tkey, tval, gate, s)
+                                     : scatter_gate<14>(c, pk, pv, tkey, tval, gate, s);
     release(pk, s);
     release(pv, s);
     release(tkey, s);
