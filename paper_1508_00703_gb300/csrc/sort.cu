@@ -135,7 +135,7 @@ int bits_for(int64_t max_key)
 //      (in the conflict build's first pass also the id checks);
 //   2. k_rs_chunk_sum / k_rs_chunk_scan / k_rs_chunk_down: the counts in
 //      digit-major order become the global output offset of each (tile,
-//      digit), computed hierarchically over chunks of 256 tiles;
+//      digit), computed hierarchically over chunks of tiles (chunk_tiles);
 //   3. k_rs_scatter: each tile ranks its pairs stably (one ballot per
 //      digit bit, per-warp running counts, prefix over warps and digits), stages
 //      them in shared memory in output order, and writes every digit's run
@@ -144,7 +144,20 @@ int bits_for(int64_t max_key)
 constexpr int RS_THREADS = 256;
 constexpr int RS_IPT = 16;
 constexpr int RS_TILE = RS_THREADS * RS_IPT;   // pairs per tile
-constexpr int RS_CHUNK = 256;                  // tiles per scan chunk
+
+// tiles per scan chunk: near the square root of their number, so that neither
+// the walk along a chunk nor the one over the chunks is long (16 to 256, and a
+// multiple of 16, which the walks load at a time).  With chunks of 256 tiles at
+// every size the three scan kernels of a pass took 41 us for 2M pairs and 31 for
+// 20M; so, and with the scan over up to 128 chunks inside the last of them, 14 and 15.
+constexpr int RS_CHUNK = 256;                  // longest; known to the compiler where it is taken
+constexpr int RS_SCAN_CHUNKS = 128;
+static int chunk_tiles(int64_t n_tiles)
+{
+    int c = 16;
+    while (c < RS_CHUNK && ((int64_t)c * c * 2 < n_tiles || (n_tiles + c - 1) / c > RS_SCAN_CHUNKS)) c *= 2;
+    return c;
+}
 
 // Per-tile digit counts.  In the first pass of the conflict build the same
 // read of the ids also checks them: each must be below `range` (else
@@ -206,14 +219,25 @@ __global__ __launch_bounds__(RS_THREADS) void k_rs_hist(const uint32_t *__restri
     }
 }
 
-// column sums of the [tile][digit] counts over each chunk of RS_CHUNK tiles (RADIX threads)
-__global__ void k_rs_chunk_sum(const uint32_t *__restrict__ hist, int64_t n_tiles, int radix,
+// column sums of the [tile][digit] counts over each chunk of tiles (RADIX threads)
+template <bool BIG>
+__global__ void k_rs_chunk_sum(const uint32_t *__restrict__ hist, int64_t n_tiles, int chunk, int radix,
                                uint32_t *__restrict__ csum, const int *status)
 {
     if (read_status(status)) return;
-    const int64_t t0 = (int64_t)blockIdx.x * RS_CHUNK, t1 = min64(n_tiles, t0 + RS_CHUNK);
+    const int64_t t0 = (int64_t)blockIdx.x * (BIG ? RS_CHUNK : chunk), t1 = min64(n_tiles, t0 + (BIG ? RS_CHUNK : chunk));
     uint32_t s = 0;
-    for (int64_t t = t0; t < t1; ++t) s += hist[t * radix + threadIdx.x];
+    if (BIG) {
+        for (int64_t t = t0; t < t1; ++t) s += hist[t * radix + threadIdx.x];
+    } else {
+        for (int64_t t = t0; t < t1; t += 16) {       // 16 loads in flight
+            uint32_t v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = t + u < t1 ? hist[(t + u) * radix + threadIdx.x] : 0u;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) s += v[u];
+        }
+    }
     csum[(int64_t)blockIdx.x * radix + threadIdx.x] = s;
 }
 
@@ -243,13 +267,42 @@ __global__ void k_rs_chunk_scan(const uint32_t *__restrict__ csum, int64_t n_chu
     }
 }
 
-// hist[tile][d] <- global output offset of digit d for that tile
-__global__ void k_rs_chunk_down(uint32_t *__restrict__ hist, int64_t n_tiles, int radix,
-                                const uint32_t *__restrict__ cbase, const int *status)
+// hist[tile][d] <- global output offset of digit d for that tile.  `base` holds
+// cbase, or (SCAN) csum, from which each block finds its chunk's cbase itself:
+// for few chunks that takes less than a launch of its own.
+template <bool SCAN>
+__global__ void k_rs_chunk_down(uint32_t *__restrict__ hist, int64_t n_tiles, int chunk, int radix,
+                                const uint32_t *__restrict__ base, int n_chunks, const int *status)
 {
     if (read_status(status)) return;
-    const int64_t t0 = (int64_t)blockIdx.x * RS_CHUNK, t1 = min64(n_tiles, t0 + RS_CHUNK);
-    uint32_t run = cbase[(int64_t)blockIdx.x * radix + threadIdx.x];
+    const int64_t t0 = (int64_t)blockIdx.x * (SCAN ? chunk : RS_CHUNK), t1 = min64(n_tiles, t0 + (SCAN ? chunk : RS_CHUNK));
+    uint32_t run = 0;
+    if (SCAN) {
+        __shared__ uint32_t wsum[32];
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        uint32_t before = 0, all = 0;             // this digit in earlier chunks, in all
+        for (int c = 0; c < n_chunks; c += 16) {
+            uint32_t v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = c + u < n_chunks ? base[(c + u) * radix + threadIdx.x] : 0u;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) {
+                all += v[u];
+                before += c + u < (int)blockIdx.x ? v[u] : 0u;
+            }
+        }
+        uint32_t x = all;
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, x, off);
+            if (lane >= off) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        run = x - all + before;
+        for (int w = 0; w < warp; ++w) run += wsum[w];
+    } else {
+        run = base[(int64_t)blockIdx.x * radix + threadIdx.x];
+    }
     for (int64_t t = t0; t < t1; t += 16) {       // 16 loads in flight, then 16 stores
         uint32_t v[16];
 #pragma unroll
@@ -429,7 +482,8 @@ int radix_passes(const uint32_t *keys_in, const int32_t *vals_in, uint32_t *keys
         if (known) configured[dev].store(true, std::memory_order_release);
     }
     const int64_t n_tiles = (n + RS_TILE - 1) / RS_TILE;
-    const int64_t n_chunks = (n_tiles + RS_CHUNK - 1) / RS_CHUNK;
+    const int chunk = chunk_tiles(n_tiles);
+    const int64_t n_chunks = (n_tiles + chunk - 1) / chunk;
     uint32_t *hist = nullptr, *csum = nullptr, *cbase = nullptr;
     int rc = alloc((void **)&hist, sizeof(uint32_t) * RADIX * n_tiles, s);
     rc = rc ? rc : alloc((void **)&csum, sizeof(uint32_t) * RADIX * n_chunks, s);
@@ -445,12 +499,20 @@ int radix_passes(const uint32_t *keys_in, const int32_t *vals_in, uint32_t *keys
             k_rs_hist<D><<<(unsigned)n_tiles, RS_THREADS, 0, s>>>(kin, n, shift, hist, p == 0 ? range : 0u,
                                                                   p == 0 ? descents : nullptr, const_cast<int *>(status));
             note_launch();
-            k_rs_chunk_sum<<<(unsigned)n_chunks, RADIX, 0, s>>>(hist, n_tiles, RADIX, csum, status);
+            const auto sum = chunk == RS_CHUNK ? k_rs_chunk_sum<true> : k_rs_chunk_sum<false>;
+            sum<<<(unsigned)n_chunks, RADIX, 0, s>>>(hist, n_tiles, chunk, RADIX, csum, status);
             note_launch();
-            k_rs_chunk_scan<<<1, RADIX, 0, s>>>(csum, n_chunks, RADIX, cbase, status);
-            note_launch();
-            k_rs_chunk_down<<<(unsigned)n_chunks, RADIX, 0, s>>>(hist, n_tiles, RADIX, cbase, status);
-            note_launch();
+            if (n_chunks <= RS_SCAN_CHUNKS) {
+                k_rs_chunk_down<true><<<(unsigned)n_chunks, RADIX, 0, s>>>(hist, n_tiles, chunk, RADIX, csum,
+                                                                           (int)n_chunks, status);
+                note_launch();
+            } else {
+                k_rs_chunk_scan<<<1, RADIX, 0, s>>>(csum, n_chunks, RADIX, cbase, status);
+                note_launch();
+                k_rs_chunk_down<false><<<(unsigned)n_chunks, RADIX, 0, s>>>(hist, n_tiles, chunk, RADIX, cbase,
+                                                                            (int)n_chunks, status);
+                note_launch();
+            }
             k_rs_scatter<D><<<(unsigned)n_tiles, RS_THREADS, smem, s>>>(kin, vin, ko, vo, n, shift, hist, status);
             note_launch();
             kin = ko;
