@@ -302,6 +302,7 @@ int block_ready_run(const pdb_csr *X, const float *y, const uint32_t *gate, floa
     const int64_t smem = block_ready_smem(X->n_cols, max_row);
     if (smem == 0) return PDB_ETOOBIG;
     const BlockReadyKernel kern = trace ? block_ready_kernel<true>(max_row, loss) : block_ready_kernel<false>(max_row, loss);
+    // (every call: another size, and another kernel per form, loss and trace)
     if (cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return PDB_ECUDA;
     // Warps: more examples in flight reach further ahead, fewer share the SM's

@@ -710,18 +710,15 @@ int ensure_gate(pdb_conflicts *c, cudaStream_t s)
     const int64_t nnz = c->nnz;
     uint32_t *gate = nullptr, *pk = nullptr, *tkey = nullptr;
     int32_t *pv = nullptr, *tval = nullptr;
+    void *scratch = nullptr;
     int rc = alloc((void **)&gate, sizeof(uint32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&pk, sizeof(uint32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&pv, sizeof(int32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&tkey, sizeof(uint32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&tval, sizeof(int32_t) * nnz, s);
+    rc = rc ? rc : alloc_block(&scratch, {{(void **)&pk, sizeof(uint32_t) * nnz}, {(void **)&pv, sizeof(int32_t) * nnz},
+                                          {(void **)&tkey, sizeof(uint32_t) * nnz},
+                                          {(void **)&tval, sizeof(int32_t) * nnz}}, s);
     if (rc == PDB_OK)
         rc = bits_for(nnz - 1) == 25 ? scatter_gate<15>(c, pk, pv, tkey, tval, gate, s)
                                      : scatter_gate<14>(c, pk, pv, tkey, tval, gate, s);
-    release(pk, s);
-    release(pv, s);
-    release(tkey, s);
-    release(tval, s);
+    release(scratch, s);
     if (rc != PDB_OK) {
         release(gate, s);
         return rc;
@@ -989,9 +986,10 @@ int pdb_build_conflicts(const pdb_csr *X, pdb_conflicts **out, void *stream)
     rc = rc ? rc : alloc((void **)&c->feat_ptr, sizeof(int64_t) * (F + 1), s);
     uint32_t *skey = nullptr, *tkey = nullptr;
     int32_t *tval = nullptr;
-    rc = rc ? rc : alloc((void **)&skey, sizeof(uint32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&tkey, sizeof(uint32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&tval, sizeof(int32_t) * nnz, s);
+    void *scratch = nullptr;
+    rc = rc ? rc : alloc_block(&scratch, {{(void **)&skey, sizeof(uint32_t) * nnz},
+                                          {(void **)&tkey, sizeof(uint32_t) * nnz},
+                                          {(void **)&tval, sizeof(int32_t) * nnz}}, s);
     c->status = c->info;
     if (rc == PDB_OK) {
         rc = fill_words(c->info, 0u, sizeof(int) * INFO_WORDS, s);
@@ -1011,9 +1009,7 @@ int pdb_build_conflicts(const pdb_csr *X, pdb_conflicts **out, void *stream)
                                                         partition ? c->gate_window : nullptr, c->info);
         note_launch();
     }
-    release(skey, s);
-    release(tkey, s);
-    release(tval, s);
+    release(scratch, s);
     if (rc == PDB_OK) rc = copy_words_to_host(c->h_info, c->info, sizeof(int) * INFO_WORDS, s);
     cudaEventRecord(c->ev1, s);
     mark_use(c, nullptr, s);
@@ -1060,8 +1056,7 @@ void pdb_schedule_free(pdb_schedule *s)
     if (!s) return;
     // the schedule's own work only: other streams of the device keep running
     if (s->ev_use) cudaEventSynchronize(s->ev_use);
-    free_ptrs({s->level, s->order, s->indeg, s->queue, s->level_ptr, s->ctl, s->rec, s->link, s->bar, s->ticket,
-               s->prog, s->wctl, s->reads, s->writes, s->rbits, s->wbits});
+    free_ptrs({s->level, s->order, s->indeg, s->queue, s->level_ptr, s->ctl, s->rec, s->link, s->bar, s->prog, s->wctl, s->reads, s->writes, s->rbits, s->wbits});
     for (cudaEvent_t e : {s->ev0, s->ev1, s->ev_use})
         if (e) cudaEventDestroy(e);
     delete s;
@@ -1102,11 +1097,12 @@ int pdb_schedule_build(const pdb_conflicts *c, pdb_sched_mode mode, pdb_schedule
     }
     const int64_t N = c->n_rows, F = c->n_cols, nnz = c->nnz;
     cudaEventRecord(h->ev0, s);
-    int rc = alloc((void **)&h->bar, sizeof(GridBarrier), s);
-    rc = rc ? rc : alloc((void **)&h->ticket, sizeof(unsigned long long), s);
+    // the grid barrier and the ticket, zeroed together
+    static_assert(sizeof(GridBarrier) <= 16, "the ticket follows the barrier");
+    int rc = alloc((void **)&h->bar, 16 + sizeof(unsigned long long), s);
     if (rc == PDB_OK) {
-        rc = fill_words(h->bar, 0u, sizeof(GridBarrier), s);
-        rc = rc ? rc : fill_words(h->ticket, 0u, sizeof(unsigned long long), s);
+        h->ticket = reinterpret_cast<unsigned long long *>(h->bar + 16 / sizeof(GridBarrier));
+        rc = fill_words(h->bar, 0u, 16 + sizeof(unsigned long long), s);
     }
     if (mode == PDB_SCHED_READY) {
         // one (weight, version) record per feature; filled from w by pdb_sgd_epoch;

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "pdb.h"
 
 namespace pdb {
@@ -26,6 +28,14 @@ int persistent_grid(const void *kernel, const pdb_opts *opts, int threads = THRE
 uint64_t timeout_ns(const pdb_opts *opts);
 int alloc(void **p, size_t bytes, cudaStream_t s);   // stream-ordered, 256-byte aligned
 void release(void *p, cudaStream_t s);
+// Several arrays of one lifetime in one allocation (an allocation costs the host
+// ~5 us, which a small build waits for): pieces 256-byte aligned, in order.
+// Returns PDB_OK with *block to release, or PDB_ENOMEM with every pointer null.
+struct Piece {
+    void **p;
+    size_t bytes;
+};
+int alloc_block(void **block, std::initializer_list<Piece> pieces, cudaStream_t s);
 cudaStream_t own_stream();                           // the library's non-blocking stream (current device)
 int bits_for(int64_t max_key);                        // bits to hold values 0..max_key (>= 1)
 int grid_1d(int64_t n);                               // blocks of 256 threads for a grid-stride loop
@@ -395,7 +405,7 @@ struct pdb_schedule {
     int64_t prog_cap;         // WINDOW: flags allocated (one per example: chunks of one example or more)
     pdb::WindowCtl *wctl;     // WINDOW: ticket and watermark
     pdb::GridBarrier *bar;    // barrier for the level-synchronous engine
-    unsigned long long *ticket;
+    unsigned long long *ticket;   // in bar's allocation
     cudaEvent_t ev0, ev1;
     cudaEvent_t ev_use;      // recorded after the last work any call enqueued on the handle
     bool timed;

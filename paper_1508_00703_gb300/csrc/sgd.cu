@@ -706,13 +706,14 @@ int bsp_sort(pdb_conflicts *c, const float *val, int64_t batch, int64_t n_batche
     if (nnz == 0) return fill_words(bptr, 0u, sizeof(int64_t) * (n_batches + 1), s);
     uint32_t *key = nullptr, *skey = nullptr, *tkey = nullptr;
     int32_t *bpos = nullptr, *tval = nullptr;
+    void *scratch = nullptr;
     int rc = ensure_row_of(c, s);
     if (n_batches > 1) {
-        rc = rc ? rc : alloc((void **)&key, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&skey, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&tkey, sizeof(uint32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&bpos, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&tval, sizeof(int32_t) * nnz, s);
+        rc = rc ? rc : alloc_block(&scratch, {{(void **)&key, sizeof(uint32_t) * nnz},
+                                              {(void **)&skey, sizeof(uint32_t) * nnz},
+                                              {(void **)&tkey, sizeof(uint32_t) * nnz},
+                                              {(void **)&bpos, sizeof(int32_t) * nnz},
+                                              {(void **)&tval, sizeof(int32_t) * nnz}}, s);
         if (rc == PDB_OK) {
             k_bsp_keys<<<grid_1d(nnz), 256, 0, s>>>(c->csc_pos, c->row_of, nnz, (uint32_t)batch, key, c->status);
             note_launch();
@@ -732,7 +733,7 @@ int bsp_sort(pdb_conflicts *c, const float *val, int64_t batch, int64_t n_batche
         note_launch();
         if (cudaPeekAtLastError() != cudaSuccess) rc = PDB_ECUDA;
     }
-    for (void *q : {(void *)key, (void *)skey, (void *)tkey, (void *)bpos, (void *)tval}) release(q, s);
+    release(scratch, s);
     return rc;
 }
 
@@ -963,13 +964,12 @@ int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, floa
         int64_t *bptr = nullptr;
         int32_t *runs = nullptr;
         uint2 *n_runs = nullptr;
-        rc = alloc((void **)&bcol, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&brow, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&bval, sizeof(float) * nnz, s);
-        rc = rc ? rc : alloc((void **)&cbuf, sizeof(float) * batch, s);
-        rc = rc ? rc : alloc((void **)&bptr, sizeof(int64_t) * (n_batches + 1), s);
-        rc = rc ? rc : alloc((void **)&runs, sizeof(int32_t) * nnz, s);
-        rc = rc ? rc : alloc((void **)&n_runs, sizeof(uint2) * n_batches, s);
+        void *block = nullptr;
+        rc = alloc_block(&block, {{(void **)&bcol, sizeof(int32_t) * nnz}, {(void **)&brow, sizeof(int32_t) * nnz},
+                                  {(void **)&bval, sizeof(float) * nnz}, {(void **)&cbuf, sizeof(float) * batch},
+                                  {(void **)&bptr, sizeof(int64_t) * (n_batches + 1)},
+                                  {(void **)&runs, sizeof(int32_t) * nnz},
+                                  {(void **)&n_runs, sizeof(uint2) * n_batches}}, s);
         int64_t max_row = 0;
         if (rc == PDB_OK) {
             if (cudaEventSynchronize(c->ev1) != cudaSuccess) {
@@ -989,9 +989,7 @@ int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, floa
                     rc = launch_apply(b, r0, r1 - r0, std::min(nnz, (r1 - r0) * max_row), sms, bptr, bcol, brow, bval,
                                       runs, n_runs, cbuf, w, cm->status, true, s);
             }
-        for (void *p : {(void *)bcol, (void *)brow, (void *)bval, (void *)cbuf, (void *)bptr, (void *)runs,
-                        (void *)n_runs})
-            release(p, s);
+        release(block, s);
     }
     cudaEventRecord(cm->ev_bsp1, s);
     cm->timed_bsp = true;

@@ -113,6 +113,23 @@ void release(void *p, cudaStream_t s)
     if (p) cudaFreeAsync(p, s);
 }
 
+int alloc_block(void **block, std::initializer_list<Piece> pieces, cudaStream_t s)
+{
+    size_t total = 0;
+    for (const Piece &q : pieces) {
+        *q.p = nullptr;
+        total += (q.bytes + 255) & ~(size_t)255;
+    }
+    const int rc = alloc(block, total, s);
+    if (rc != PDB_OK) return rc;
+    char *at = (char *)*block;
+    for (const Piece &q : pieces) {
+        *q.p = at;
+        at += (q.bytes + 255) & ~(size_t)255;
+    }
+    return PDB_OK;
+}
+
 static std::atomic<long long> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
@@ -485,9 +502,10 @@ int radix_passes(const uint32_t *keys_in, const int32_t *vals_in, uint32_t *keys
     const int chunk = chunk_tiles(n_tiles);
     const int64_t n_chunks = (n_tiles + chunk - 1) / chunk;
     uint32_t *hist = nullptr, *csum = nullptr, *cbase = nullptr;
-    int rc = alloc((void **)&hist, sizeof(uint32_t) * RADIX * n_tiles, s);
-    rc = rc ? rc : alloc((void **)&csum, sizeof(uint32_t) * RADIX * n_chunks, s);
-    rc = rc ? rc : alloc((void **)&cbase, sizeof(uint32_t) * RADIX * n_chunks, s);
+    void *block = nullptr;
+    const int rc = alloc_block(&block, {{(void **)&hist, sizeof(uint32_t) * RADIX * n_tiles},
+                                        {(void **)&csum, sizeof(uint32_t) * RADIX * n_chunks},
+                                        {(void **)&cbase, sizeof(uint32_t) * RADIX * n_chunks}}, s);
     if (rc == PDB_OK) {
         const uint32_t *kin = keys_in;
         const int32_t *vin = vals_in;
@@ -519,9 +537,7 @@ int radix_passes(const uint32_t *keys_in, const int32_t *vals_in, uint32_t *keys
             vin = vo;
         }
     }
-    release(hist, s);
-    release(csum, s);
-    release(cbase, s);
+    release(block, s);
     if (rc != PDB_OK) return rc;
     return cudaPeekAtLastError() == cudaSuccess ? PDB_OK : PDB_ECUDA;
 }
