@@ -88,7 +88,10 @@ __device__ __forceinline__ bool keep_waiting(unsigned &spins, uint64_t t0, int *
 // to 512 ns 4.0-6.2 ms over boxes, 4 ns per missing count 3.0, 8 ns 2.2, 12 ns
 // 1.6; the results differ by what two runs of one form differ by (which
 // examples are in flight is the same; fewer warps would be faster still, down to
-// 0.9 ms, with reads less stale).
+// 0.9 ms, with reads less stale).  At small delays few counts are missing but each
+// takes a whole hop: a poll that finds no progress doubles the nap, from 64 to
+// 512 ns (1M such examples, delay 16: doubling alone 783 ms, both 522; delay 128:
+// 154 and 94).
 constexpr long long WAIT_NS = 12;
 __device__ __forceinline__ bool wait_count(const unsigned *counter, long long need, int *status, uint64_t timeout)
 {
@@ -97,11 +100,15 @@ __device__ __forceinline__ bool wait_count(const unsigned *counter, long long ne
     if (have >= need) return true;
     const uint64_t t0 = globaltimer();
     unsigned spins = 0;
+    long long nap = 0;
     for (;;) {
-        const long long nap = (need - have) * WAIT_NS;
+        const long long lacks = (need - have) * WAIT_NS;
+        nap = lacks > nap ? lacks : nap;
         __nanosleep(nap < 32 ? 32u : nap > 8192 ? 8192u : (unsigned)nap);
+        const long long was = have;
         have = ld_acquire_u32(counter);
         if (have >= need) return true;
+        nap = have > was ? 0 : nap < 32 ? 64 : nap < 256 ? 2 * nap : 512;
         if (!keep_waiting(spins, t0, status, timeout)) return false;
     }
 }
