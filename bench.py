@@ -360,7 +360,7 @@ def run_ours(args, rank, world, local_rank):
     resolved = int(phases[0]["sched_mode"])
     if args.delay is not None:
         resolved = -2
-    kname = {pdb.PDB_SCHED_READY: "k_sgd_ready", pdb.PDB_SCHED_LEVELS: "k_sgd_levels", -1: "k_bsp", -2: "k_sgd_ssp",
+    kname = {pdb.PDB_SCHED_READY: "k_sgd_ready", pdb.PDB_SCHED_LEVELS: "k_sgd_levels", -1: "k_bsp_apply", -2: "k_sgd_ssp",
              pdb.PDB_SCHED_CHAIN: "k_sgd_chain", pdb.PDB_SCHED_WINDOW: "k_sgd_window"}[resolved]
     roofline = {"kernel": kname,
                 "bound": "hbm", "achieved": round(sgd_gbs, 1), "peak": peak, "unit": "GB/s",
@@ -418,7 +418,7 @@ def run_ours(args, rank, world, local_rank):
                                    "loss": {0: "logistic", 1: "squared", 2: "hinge"}[p.loss]}
         del c, s, c2, s2
     if batch:
-        roofline["kernel"] = "k_bsp (whole pdb_bsp_epoch call per epoch: batch sort, gather, cooperative kernel)"
+        roofline["kernel"] = "k_bsp_apply (whole pdb_bsp_epoch call per epoch: batch sort, gather, run lists, two launches per batch)"
         result["metric"] = METRIC.replace("serially-equivalent sparse SGD", f"BSP mini-batch ({batch}) SGD")
         del result["sgd_only"]
         result["bsp_only"] = {"value": units / (ms_sgd / 1e3), "unit": UNIT}
