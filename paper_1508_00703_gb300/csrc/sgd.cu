@@ -607,7 +607,10 @@ __global__ __launch_bounds__(256, 5) void k_bsp_coef(int64_t r0, int64_t r1, con
                            const int *status)
 {
     launch_next();
-    if (read_status(status)) return;
+    if (read_status(status)) {
+        wait_previous();        // a kernel that is done leaves nothing before it running
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -637,7 +640,10 @@ __global__ __launch_bounds__(BSP_THREADS, BSP_BLOCKS) void k_bsp_apply(
 {
     __shared__ __align__(16) float s_buf[2][BSP_STAGE];
     launch_next();
-    if (read_status(status)) return;
+    if (read_status(status)) {
+        wait_previous();        // as in k_bsp_coef
+        return;
+    }
     const int64_t s0 = bptr[bi], s1 = bptr[bi + 1];
     const uint2 n = n_runs[bi];
     const BspPairs P = {(uint32_t)s1, r0, rows, bcol, brow, bval, coef};
