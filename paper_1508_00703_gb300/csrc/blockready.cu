@@ -207,10 +207,15 @@ __global__ __launch_bounds__(BR_WARPS * 32, 1) void k_sgd_block_ready(int32_t n_
             }
             return combine_group<LPE>(acc);
         };
-        // the running groups' stores, and their next examples
-        auto finish = [&](float c, bool done) {
+        // the running groups' stores, and their next examples; `seen`: when their weights
+        // had all been read, in this pass (also those of a group set aside, whose records
+        // are read again in each)
+        auto finish = [&](float c, bool done, uint64_t seen) {
             if (TRACE) {
-                if (done && sl == 0) trace[2 * (int64_t)ctg] = trace[2 * (int64_t)ctg + 1] = globaltimer();
+                if (done && sl == 0) {
+                    trace[2 * (int64_t)ctg] = seen;
+                    trace[2 * (int64_t)ctg + 1] = globaltimer();
+                }
                 __syncwarp();            // before any write is visible
             }
 #pragma unroll
@@ -225,11 +230,12 @@ __global__ __launch_bounds__(BR_WARPS * 32, 1) void k_sgd_block_ready(int32_t n_
         };
         if (run) {
             spins = 0;
+            const uint64_t seen = TRACE ? globaltimer() : 0;
             bool redo = false;
             const float c = dev_step_fast(LOSS, margin(), yc, eta, redo);
             const bool mine = run >> lane & 1u;
             if (LOSS == PDB_LOSS_LOGISTIC) slow = mine ? redo : slow;     // set aside
-            finish(c, mine && !redo);
+            finish(c, mine && !redo, seen);
             continue;
         }
         if (LOSS == PDB_LOSS_LOGISTIC) {
@@ -238,10 +244,11 @@ __global__ __launch_bounds__(BR_WARPS * 32, 1) void k_sgd_block_ready(int32_t n_
             run = __ballot_sync(FULL, slow) & alive;
             if (run) {
                 spins = 0;
+                const uint64_t seen = TRACE ? globaltimer() : 0;
                 const float c = __fmul_rn(eta, dev_grad(LOSS, margin(), yc));
                 const bool mine = run >> lane & 1u;
                 slow = mine ? false : slow;
-                finish(c, mine);
+                finish(c, mine, seen);
                 continue;
             }
         }

@@ -9,6 +9,7 @@ import pytest
 
 import oracle
 import synthdata
+from oracle import history
 
 torch = pytest.importorskip("torch")
 pdb = pytest.importorskip("paper_1508_00703_gb300")
@@ -60,3 +61,35 @@ def test_general_derivative(k):
 
 def test_largest_feature_count():
     _equal(synthdata.generate("tiny", n_rows=4000, n_cols=28000, k=12, seed=8))
+
+
+def _wild(k):
+    """Margins and labels of which a part takes the general derivative."""
+    p = synthdata.generate("tiny", n_rows=900, n_cols=500, k=k, epochs=2, seed=2)
+    rng = np.random.default_rng(k)
+    p.val = np.where(np.repeat(rng.random(p.n_rows) < 0.3, k), p.val * np.float32(3000.0), p.val).astype(np.float32)
+    return p
+
+
+@pytest.mark.parametrize("wild", [False, True])
+@pytest.mark.parametrize("k", [5, 13, 30, 60])
+def test_trace_stamps_the_reads_when_the_weights_arrived(k, wild):
+    # two moments per example, as the interface says: between them lie the margin,
+    # the combine and the derivative (more than 100 ns), so over many examples the
+    # timer has to tick between the two of some, also of those taken by the
+    # general derivative.  One time for both would hide a read made too early.
+    p = _wild(k) if wild else synthdata.generate("tiny", n_rows=6000, n_cols=3000, k=k, epochs=2, seed=k)
+    X = pdb.Csr.from_problem(p)
+    y = torch.from_numpy(p.y).cuda()
+    c = pdb.pdb_build_conflicts(X)
+    s = pdb.pdb_schedule_build(c, pdb.PDB_SCHED_READY)
+    w = torch.zeros(p.n_cols, dtype=torch.float32, device="cuda")
+    trace = torch.zeros(2 * p.epochs * p.n_rows, dtype=torch.int64, device="cuda")
+    pdb.pdb_sgd_epoch(X, y, c, s, w, p.loss, p.eta, p.epochs, opts=dict(trace=trace))
+    pdb.check_status(c)
+    assert np.array_equal(w.cpu().numpy().view(np.uint32), oracle.sgd(p).view(np.uint32))
+    tr = trace.cpu().numpy().reshape(-1, 2)
+    assert np.all(tr > 0)
+    v = history.trace_order_violations(p.row_ptr, p.col, p.epochs, tr)
+    assert v["self"] == 0 and v["rc"] == 0, v
+    assert np.mean(tr[:, 0] < tr[:, 1]) > 0.02
