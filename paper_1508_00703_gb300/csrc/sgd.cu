@@ -633,6 +633,10 @@ __global__ __launch_bounds__(256, 5) void k_bsp_coef(int64_t r0, int64_t r1, con
 // dense examples of 960 features 37 us per batch against 113.  One warp doing
 // both loads and additions took 6 cycles per term alone and 13 with every SM
 // doing so.
+//
+// The weights are read and written through L2 only, never a line kept in L1:
+// this block may already sit on an SM while blocks of the batch before there
+// still read and write other weights of the same lines.
 __global__ __launch_bounds__(BSP_THREADS, BSP_BLOCKS) void k_bsp_apply(
     int64_t bi, const int64_t *__restrict__ bptr, int32_t r0, int32_t rows, const int32_t *__restrict__ bcol,
     const int32_t *__restrict__ brow, const float *__restrict__ bval, const int32_t *__restrict__ runs,
@@ -654,7 +658,7 @@ __global__ __launch_bounds__(BSP_THREADS, BSP_BLOCKS) void k_bsp_apply(
         const float delta = block_run_sum(P, q, len, s_buf, bad);
         if (threadIdx.x == 0) {
             const int32_t j = bcol[q];
-            w[j] = __fsub_rn(w[j], delta);
+            __stcg(w + j, __fsub_rn(__ldcg(w + j), delta));
         }
     }
     wait_previous();
@@ -667,7 +671,7 @@ __global__ __launch_bounds__(BSP_THREADS, BSP_BLOCKS) void k_bsp_apply(
             float delta = 0.0f;
             if (thread_run_chunk<2>(P, j, q, delta, bad))
                 while (thread_run_chunk<4>(P, j, q, delta, bad)) {}
-            w[j] = __fsub_rn(w[j], delta);
+            __stcg(w + j, __fsub_rn(__ldcg(w + j), delta));
         }
     if (bad) set_status(status, PDB_EFAULT);   // cannot happen with a consistent batch order
 }

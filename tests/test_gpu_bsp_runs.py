@@ -70,3 +70,13 @@ def test_batches_without_nonzeros():
     p = synthdata.from_arrays(np.r_[0, np.cumsum(lens)], col, rng.standard_normal(col.size), np.ones(n), n_cols=9)
     for batch in (1, 10, 30, 90):
         _equal(p, batch)
+
+
+@pytest.mark.parametrize("batch", [8, 40, 130])
+def test_neighbouring_weights_over_overlapping_batches(batch):
+    # 70 features, so a few 128-byte lines of weights, each updated by many blocks
+    # (runs summed by threads at 8 rows a batch, by blocks above) in every one of
+    # hundreds of batches whose launches overlap: a line that a block kept in its
+    # L1 from the batch before would give a stale weight
+    p = synthdata.generate("tiny", n_rows=2600, n_cols=70, k=50, seed=batch)
+    _equal(p, batch, epochs=3)
