@@ -155,7 +155,8 @@ typedef enum {
 /* Launch and wait options; a zeroed struct (or NULL) selects the defaults. */
 typedef struct {
     int32_t blocks_per_sm;     /* persistent grid = blocks_per_sm x #SM (at most the occupancy
-                                  maximum); 0 = that maximum, for WINDOW 3, for READY 2 or 4 */
+                                  maximum); 0 = that maximum, for WINDOW 3, for READY 2 or 4;
+                                  pdb_bsp_epoch: the most blocks of one launch, 0 = no limit */
     int32_t ticket_chunk;      /* READY: consecutive examples a warp takes per ticket; 0 = 1 or 2 by
                                   how often examples conflict, under pdb_ssp_epoch 2 */
     double wait_timeout_s;     /* limit of every device-side wait; 0 = 2 seconds; at most 10^6 seconds */
@@ -328,8 +329,10 @@ int pdb_ssp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, cons
  * dloss/dm at the weights of the batch start (read barrier), then each
  * feature j takes delta_j = sum over the batch's examples, ascending, of
  * c_i * x_ij and w_j = w_j - delta_j (write barrier).  batch = 1 equals
- * sequential SGD (Theorem 1).  Two kernel launches per batch (no wait inside a
- * kernel: opts->blocks_per_sm and wait_timeout_s play no part).  Allocates
+ * sequential SGD (Theorem 1).  Two kernel launches per batch, of at most
+ * opts->blocks_per_sm blocks per SM each when that is set (and then no launch
+ * overlaps the one before it; 0 = each kernel's own grid).  No kernel waits for
+ * another's memory, so opts->wait_timeout_s has nothing to limit.  Allocates
  * per-call scratch stream-ordered and waits (host) for the conflict build of c
  * to finish. */
 int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, float *w, pdb_loss loss, float eta,

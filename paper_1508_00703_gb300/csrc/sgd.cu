@@ -749,7 +749,8 @@ int bsp_sort(pdb_conflicts *c, const float *val, int64_t batch, int64_t n_batche
 
 // the two launches of a batch; `follow`: the launch before on this stream is
 // this batch's or the batch before's other one, and this kernel may start while
-// it drains (launch_next, wait_previous)
+// it drains (launch_next, wait_previous).  `most`: the largest grid (0: any; both
+// kernels stride over their work).
 struct BspLaunch {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr = {};
@@ -765,9 +766,10 @@ struct BspLaunch {
     }
 };
 int launch_coef(int64_t r0, int64_t r1, const pdb_csr *X, const float *y, const float *w, int loss, float eta,
-                float *coef, const int *status, bool follow, cudaStream_t s)
+                float *coef, const int *status, bool follow, int64_t most, cudaStream_t s)
 {
-    const BspLaunch l(grid_1d((r1 - r0) * 32), 256, follow, s);
+    const int64_t blocks = grid_1d((r1 - r0) * 32);
+    const BspLaunch l(most > 0 ? std::min(blocks, most) : blocks, 256, follow, s);
     const cudaError_t e = cudaLaunchKernelEx(&l.cfg, k_bsp_coef, r0, r1, X->row_ptr, X->col, X->val, y, w, loss, eta,
                                              coef, status);
     note_launch();
@@ -776,11 +778,12 @@ int launch_coef(int64_t r0, int64_t r1, const pdb_csr *X, const float *y, const 
 // pairs: at least the number of the batch's pairs
 int launch_apply(int64_t bi, int64_t r0, int64_t rows, int64_t pairs, int sms, const int64_t *bptr, const int32_t *bcol,
                  const int32_t *brow, const float *bval, const int32_t *runs, const uint2 *n_runs, const float *coef,
-                 float *w, int *status, bool follow, cudaStream_t s)
+                 float *w, int *status, bool follow, int64_t most, cudaStream_t s)
 {
     // a long run holds more than BSP_LONG pairs, so this covers one block per long run up to the cap
+    if (most <= 0) most = (int64_t)sms * BSP_BLOCKS;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((pairs + BSP_LONG - 1) / BSP_LONG,
-                                                                  (int64_t)sms * BSP_BLOCKS));
+                                                                  std::min<int64_t>(most, (int64_t)sms * BSP_BLOCKS)));
     const BspLaunch l(blocks, BSP_THREADS, follow, s);
     const cudaError_t e = cudaLaunchKernelEx(&l.cfg, k_bsp_apply, bi, bptr, (int32_t)r0, (int32_t)rows, bcol, brow,
                                              bval, runs, n_runs, coef, w, status);
@@ -990,14 +993,19 @@ int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, floa
         }
         rc = rc ? rc : bsp_sort(cm, X->val, batch, n_batches, bcol, brow, bval, bptr, runs, n_runs, s);
         const int sms = launch_info().sms;
-        // the first launch waits for everything before it; the others start early
+        // blocks_per_sm caps what the call keeps resident: each grid, and no kernel
+        // beside the one before it.  Otherwise the first launch waits for everything
+        // before it, and the others start early.
+        const bool capped = opts && opts->blocks_per_sm > 0;
+        const int64_t most = capped ? (int64_t)opts->blocks_per_sm * sms : 0;
         for (int ep = 0; rc == PDB_OK && ep < n_epochs; ++ep)
             for (int64_t b = 0; rc == PDB_OK && b < n_batches; ++b) {
                 const int64_t r0 = b * batch, r1 = std::min(N, r0 + batch);
-                rc = launch_coef(r0, r1, X, y, w, (int)loss, eta, cbuf, cm->status, ep > 0 || b > 0, s);
+                rc = launch_coef(r0, r1, X, y, w, (int)loss, eta, cbuf, cm->status, !capped && (ep > 0 || b > 0),
+                                 most, s);
                 if (rc == PDB_OK && nnz > 0)
                     rc = launch_apply(b, r0, r1 - r0, std::min(nnz, (r1 - r0) * max_row), sms, bptr, bcol, brow, bval,
-                                      runs, n_runs, cbuf, w, cm->status, true, s);
+                                      runs, n_runs, cbuf, w, cm->status, !capped, most, s);
             }
         release(block, s);
     }
@@ -1070,7 +1078,7 @@ int pdb_bsp_coef(const pdb_bsp_plan *p, const pdb_csr *X, const float *y, const 
     if (row_end > row_begin && row_begin / p->batch != (row_end - 1) / p->batch) return PDB_EINVAL;
     if (row_end == row_begin) return PDB_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    rc = launch_coef(row_begin, row_end, X, y, w, (int)loss, eta, coef, p->c->status, false, s);
+    rc = launch_coef(row_begin, row_end, X, y, w, (int)loss, eta, coef, p->c->status, false, 0, s);
     return rc == PDB_OK && cudaPeekAtLastError() == cudaSuccess ? PDB_OK : PDB_ECUDA;
 }
 
@@ -1086,7 +1094,7 @@ int pdb_bsp_apply(const pdb_bsp_plan *p, float *w, int64_t batch_index, const fl
     const int64_t r0 = batch_index * p->batch, rows = std::min(p->c->n_rows, r0 + p->batch) - r0;
     cudaStream_t s = (cudaStream_t)stream;
     const int rc = launch_apply(batch_index, r0, rows, s1 - s0, launch_info().sms, p->bptr, p->bcol, p->brow, p->bval,
-                                p->runs, p->n_runs, coef, w, const_cast<pdb_conflicts *>(p->c)->status, false, s);
+                                p->runs, p->n_runs, coef, w, const_cast<pdb_conflicts *>(p->c)->status, false, 0, s);
     if (p->ev_use) cudaEventRecord(p->ev_use, s);
     return rc == PDB_OK && cudaPeekAtLastError() == cudaSuccess ? PDB_OK : PDB_ECUDA;
 }

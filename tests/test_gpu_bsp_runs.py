@@ -23,14 +23,14 @@ def _cuda():
     pdb.load()
 
 
-def _equal(p, batch, epochs=2):
+def _equal(p, batch, epochs=2, opts=None):
     p.epochs = epochs
     X = pdb.Csr.from_problem(p)
     y = torch.from_numpy(p.y).cuda()
     c = pdb.pdb_build_conflicts(X)
     ref = oracle.bsp(p, batch).view(np.uint32)
     w = torch.zeros(p.n_cols, dtype=torch.float32, device="cuda")
-    pdb.pdb_bsp_epoch(X, y, c, w, p.loss, p.eta, batch, epochs)
+    pdb.pdb_bsp_epoch(X, y, c, w, p.loss, p.eta, batch, epochs, opts=opts)
     pdb.check_status(c)
     assert np.array_equal(w.cpu().numpy().view(np.uint32), ref)
     w.zero_()
@@ -80,3 +80,39 @@ def test_neighbouring_weights_over_overlapping_batches(batch):
     # L1 from the batch before would give a stale weight
     p = synthdata.generate("tiny", n_rows=2600, n_cols=70, k=50, seed=batch)
     _equal(p, batch, epochs=3)
+
+
+@pytest.mark.parametrize("per_sm", [1, 2, 1000])
+def test_blocks_per_sm_keeps_the_result(per_sm):
+    # grids smaller than the work: rows, long runs and short runs by strides
+    _equal(_head(9000, cols=30000), 9000, opts=dict(blocks_per_sm=per_sm))
+    _equal(synthdata.generate("tiny", n_rows=3000, n_cols=3000, k=60, seed=1), 1500, opts=dict(blocks_per_sm=per_sm))
+
+
+def test_blocks_per_sm_limits_the_grid():
+    # margins bound by the latency of random reads: one block of 8 warps per SM
+    # takes several times as long as the 5 that fit (measured 0.77 against 0.17 ms)
+    n, k, cols = 300_000, 32, 4_000_000
+    g = torch.Generator(device="cuda").manual_seed(1)
+    at = torch.arange(k, device="cuda") * (cols // k)
+    col = (torch.randint(0, cols // k, (n, k), device="cuda", generator=g) + at).int().reshape(-1)
+    X = pdb.Csr(torch.arange(n + 1, device="cuda") * k, col, torch.randn(n * k, device="cuda", generator=g), cols)
+    y = torch.randn(n, device="cuda", generator=g)
+    c = pdb.pdb_build_conflicts(X)
+    w = torch.zeros(cols, device="cuda")
+
+    def ms(opts, epochs):
+        times = []
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            pdb.pdb_bsp_epoch(X, y, c, w, pdb.PDB_LOSS_SQUARED, 1e-6, n, epochs, opts=opts)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return min(times)
+
+    def per_epoch(opts):
+        return ms(opts, 11) - ms(opts, 1)
+    assert per_epoch(dict(blocks_per_sm=1)) > 2 * per_epoch(None)
+    pdb.check_status(c)
