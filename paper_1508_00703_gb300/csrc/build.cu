@@ -710,9 +710,9 @@ int ensure_gate(pdb_conflicts *c, cudaStream_t s)
     const int64_t nnz = c->nnz;
     uint32_t *gate = nullptr, *pk = nullptr, *tkey = nullptr;
     int32_t *pv = nullptr, *tval = nullptr;
-    void *scratch = nullptr;
+    Block scratch;
     int rc = alloc((void **)&gate, sizeof(uint32_t) * nnz, s);
-    rc = rc ? rc : alloc_block(&scratch, {{(void **)&pk, sizeof(uint32_t) * nnz}, {(void **)&pv, sizeof(int32_t) * nnz},
+    rc = rc ? rc : alloc_block(scratch, {{(void **)&pk, sizeof(uint32_t) * nnz}, {(void **)&pv, sizeof(int32_t) * nnz},
                                           {(void **)&tkey, sizeof(uint32_t) * nnz},
                                           {(void **)&tval, sizeof(int32_t) * nnz}}, s);
     if (rc == PDB_OK)
@@ -986,8 +986,8 @@ int pdb_build_conflicts(const pdb_csr *X, pdb_conflicts **out, void *stream)
     rc = rc ? rc : alloc((void **)&c->feat_ptr, sizeof(int64_t) * (F + 1), s);
     uint32_t *skey = nullptr, *tkey = nullptr;
     int32_t *tval = nullptr;
-    void *scratch = nullptr;
-    rc = rc ? rc : alloc_block(&scratch, {{(void **)&skey, sizeof(uint32_t) * nnz},
+    Block scratch;
+    rc = rc ? rc : alloc_block(scratch, {{(void **)&skey, sizeof(uint32_t) * nnz},
                                           {(void **)&tkey, sizeof(uint32_t) * nnz},
                                           {(void **)&tval, sizeof(int32_t) * nnz}}, s);
     c->status = c->info;

@@ -716,10 +716,10 @@ int bsp_sort(pdb_conflicts *c, const float *val, int64_t batch, int64_t n_batche
     if (nnz == 0) return fill_words(bptr, 0u, sizeof(int64_t) * (n_batches + 1), s);
     uint32_t *key = nullptr, *skey = nullptr, *tkey = nullptr;
     int32_t *bpos = nullptr, *tval = nullptr;
-    void *scratch = nullptr;
+    Block scratch;
     int rc = ensure_row_of(c, s);
     if (n_batches > 1) {
-        rc = rc ? rc : alloc_block(&scratch, {{(void **)&key, sizeof(uint32_t) * nnz},
+        rc = rc ? rc : alloc_block(scratch, {{(void **)&key, sizeof(uint32_t) * nnz},
                                               {(void **)&skey, sizeof(uint32_t) * nnz},
                                               {(void **)&tkey, sizeof(uint32_t) * nnz},
                                               {(void **)&bpos, sizeof(int32_t) * nnz},
@@ -977,8 +977,8 @@ int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, floa
         int64_t *bptr = nullptr;
         int32_t *runs = nullptr;
         uint2 *n_runs = nullptr;
-        void *block = nullptr;
-        rc = alloc_block(&block, {{(void **)&bcol, sizeof(int32_t) * nnz}, {(void **)&brow, sizeof(int32_t) * nnz},
+        Block block;
+        rc = alloc_block(block, {{(void **)&bcol, sizeof(int32_t) * nnz}, {(void **)&brow, sizeof(int32_t) * nnz},
                                   {(void **)&bval, sizeof(float) * nnz}, {(void **)&cbuf, sizeof(float) * batch},
                                   {(void **)&bptr, sizeof(int64_t) * (n_batches + 1)},
                                   {(void **)&runs, sizeof(int32_t) * nnz},

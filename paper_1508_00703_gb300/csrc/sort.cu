@@ -113,16 +113,37 @@ void release(void *p, cudaStream_t s)
     if (p) cudaFreeAsync(p, s);
 }
 
-int alloc_block(void **block, std::initializer_list<Piece> pieces, cudaStream_t s)
+static constexpr size_t BLOCK_BYTES = 32 << 20;
+
+void release(const Block &b, cudaStream_t s)
+{
+    for (int i = 0; i < b.n; ++i) release(b.own[i], s);
+}
+
+int alloc_block(Block &b, std::initializer_list<Piece> pieces, cudaStream_t s)
 {
     size_t total = 0;
     for (const Piece &q : pieces) {
         *q.p = nullptr;
         total += (q.bytes + 255) & ~(size_t)255;
     }
-    const int rc = alloc(block, total, s);
+    if (total > BLOCK_BYTES && pieces.size() <= sizeof(b.own) / sizeof(b.own[0])) {
+        for (const Piece &q : pieces) {
+            const int rc = alloc(q.p, q.bytes, s);
+            if (rc != PDB_OK) {
+                release(b, s);
+                b.n = 0;
+                for (const Piece &r : pieces) *r.p = nullptr;
+                return rc;
+            }
+            b.own[b.n++] = *q.p;
+        }
+        return PDB_OK;
+    }
+    const int rc = alloc(&b.own[0], total, s);
     if (rc != PDB_OK) return rc;
-    char *at = (char *)*block;
+    b.n = 1;
+    char *at = (char *)b.own[0];
     for (const Piece &q : pieces) {
         *q.p = at;
         at += (q.bytes + 255) & ~(size_t)255;
@@ -502,8 +523,8 @@ int radix_passes(const uint32_t *keys_in, const int32_t *vals_in, uint32_t *keys
     const int chunk = chunk_tiles(n_tiles);
     const int64_t n_chunks = (n_tiles + chunk - 1) / chunk;
     uint32_t *hist = nullptr, *csum = nullptr, *cbase = nullptr;
-    void *block = nullptr;
-    const int rc = alloc_block(&block, {{(void **)&hist, sizeof(uint32_t) * RADIX * n_tiles},
+    Block block;
+    const int rc = alloc_block(block, {{(void **)&hist, sizeof(uint32_t) * RADIX * n_tiles},
                                         {(void **)&csum, sizeof(uint32_t) * RADIX * n_chunks},
                                         {(void **)&cbase, sizeof(uint32_t) * RADIX * n_chunks}}, s);
     if (rc == PDB_OK) {
