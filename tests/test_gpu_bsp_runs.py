@@ -116,3 +116,16 @@ def test_blocks_per_sm_limits_the_grid():
         return ms(opts, 11) - ms(opts, 1)
     assert per_epoch(dict(blocks_per_sm=1)) > 2 * per_epoch(None)
     pdb.check_status(c)
+
+
+@pytest.mark.parametrize("turns", [1, 2, 3])
+def test_many_short_runs(turns):
+    # as many runs of one term as one turn of the apply grid's threads takes, and one
+    # fewer and more; then two and three turns (a thread holds two runs at once)
+    step = torch.cuda.get_device_properties(0).multi_processor_count * 8 * 128
+    for n in (turns * step - 1, turns * step, turns * step + 1):
+        rng = np.random.default_rng(n)
+        row_ptr = np.minimum(np.arange((n + 63) // 64 + 1) * 64, n)
+        p = synthdata.from_arrays(row_ptr, np.arange(n), rng.standard_normal(n).astype(np.float32),
+                                  rng.standard_normal(len(row_ptr) - 1), n_cols=n + 3, loss="squared", eta=0.01)
+        _equal(p, p.n_rows, epochs=1)
