@@ -544,86 +544,117 @@ __device__ __forceinline__ void short_runs(const BspPairs &P, const int32_t *__r
 // and the length, two words each, backwards from runs[bptr[b + 1] - 1] (a long
 // run has more than two pairs, so the two lists never meet); counts in n_runs[b]
 // (short, long; zeroed before).  skey: the batch of each pair (null: one batch).
-__global__ void k_bsp_runs(const uint32_t *__restrict__ skey, const int32_t *__restrict__ bcol,
+// A block's turn is a chain of waits (pairs, bounds, places), so what bounds this is
+// how much one warp has in flight and how little it loads: each pair's feature once,
+// its neighbours' by shuffles.  20M pairs in one batch / in seven: 97 / 109 us with
+// six loads per pair and a reservation per warp, 48 / 52 so (four blocks per SM; five
+// or more spill).
+static_assert(BSP_LONG == 16, "the pair a long run's length ahead is in the other half of the warp");
+__global__ __launch_bounds__(256, 4) void k_bsp_runs(const uint32_t *__restrict__ skey, const int32_t *__restrict__ bcol,
                            const int64_t *__restrict__ bptr, int64_t nnz, int32_t *__restrict__ runs, uint2 *n_runs,
                            const int *status)
 {
     if (read_status(status)) return;
-    constexpr int E = 8;                // 256 pairs per warp and reservation: one address takes few atomics
-    const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * E;
-    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane) * E; base < nnz; base += stride) {
-        int32_t j[E], before[E], far[E];
-        uint32_t bt[E], bt_before[E], bt_far[E];
+    constexpr int E = 8;                // 256 pairs per warp and turn
+    __shared__ unsigned s_n[2][8];      // short and long runs of the block's warps, then where each puts its own
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t n = (uint32_t)nnz, stride = gridDim.x * 256u * E;       // (no overflow: n < 2^31, stride < 2^24)
+    for (uint32_t base0 = blockIdx.x * 256u * E; base0 < n; base0 += stride) {
+        const uint32_t base = base0 + (uint32_t)warp * 32u * E;
+        // the features of the warp's pairs, of the one before them and of the 16 after
+        int32_t j[E + 1], prev = base > 0 && base <= n ? bcol[base - 1] : -1;
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int64_t s = base + 32 * e + lane, f = s + BSP_LONG;
-            j[e] = s < nnz ? bcol[s] : -1;
-            before[e] = s > 0 && s < nnz ? bcol[s - 1] : -1;
-            far[e] = f < nnz ? bcol[f] : -1;
-            bt[e] = s < nnz && skey ? skey[s] : 0u;
-            bt_before[e] = s > 0 && s < nnz && skey ? skey[s - 1] : 0u;
-            bt_far[e] = f < nnz && skey ? skey[f] : 0u;
+        for (int e = 0; e <= E; ++e) {
+            const uint32_t s = base + 32u * e + lane;
+            j[e] = s < n && (e < E || lane < BSP_LONG) ? bcol[s] : -1;
         }
-        unsigned sm[E], lm[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const bool start = j[e] >= 0 && (before[e] != j[e] || bt_before[e] != bt[e]);
-            const bool is_long = start && far[e] == j[e] && bt_far[e] == bt[e];
-            sm[e] = __ballot_sync(FULL, start && !is_long);
-            lm[e] = __ballot_sync(FULL, is_long);
-        }
-        // the batches of these pairs, one after the other (nearly always one)
-        const uint32_t b_first = __shfl_sync(FULL, bt[0], 0);
-        uint32_t b_last = 0;
-        {
-            const int64_t last = min64(nnz, base + 32 * E) - 1;
-            b_last = skey ? skey[last] : 0u;
-        }
+        // the batches of the warp's pairs, one after the other.  A block whose pairs are
+        // all of one batch (nearly always) reserves its places in the lists at once, since
+        // a batch's counter is one address.
+        const bool one_batch = !skey || skey[base0] == skey[min(n, base0 + 256u * E) - 1];
+        const uint32_t b_first = skey ? skey[one_batch ? base0 : min(base, n - 1)] : 0u;
+        const uint32_t b_last = one_batch ? b_first : skey[min(n, base + 32u * E) - 1];
         for (uint32_t bb = b_first; bb <= b_last; ++bb) {
-            int n_s = 0, n_l = 0;
-            unsigned ms[E], ml[E];
+            const uint32_t b0 = (uint32_t)bptr[bb], b1 = (uint32_t)bptr[bb + 1];
+            unsigned sm[E], lm[E], n_s = 0, n_l = 0;
+            int32_t last = prev, half = __shfl_xor_sync(FULL, j[0], BSP_LONG);
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                const unsigned mine = __ballot_sync(FULL, bt[e] == bb);
-                ms[e] = sm[e] & mine;
-                ml[e] = lm[e] & mine;
-                n_s += __popc(ms[e]);
-                n_l += __popc(ml[e]);
+                const uint32_t s = base + 32u * e + lane;
+                const int32_t turn = __shfl_sync(FULL, j[e], (lane + 31) & 31), next = __shfl_xor_sync(FULL, j[e + 1], BSP_LONG);
+                const int32_t before = lane ? turn : last, far = lane < BSP_LONG ? half : next;
+                last = turn;                   // lane 0: the last of these 32
+                half = next;
+                const bool start = s >= b0 && s < b1 && (s == b0 || before != j[e]);
+                const bool is_long = start && s + BSP_LONG < b1 && far == j[e];
+                sm[e] = __ballot_sync(FULL, start && !is_long);
+                lm[e] = __ballot_sync(FULL, is_long);
+            }
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                n_s += __popc(sm[e]);
+                n_l += __popc(lm[e]);
             }
             unsigned at_s = 0, at_l = 0;
-            if (lane == 0 && n_s) at_s = atomicAdd(&n_runs[bb].x, (unsigned)n_s);
-            if (lane == 0 && n_l) at_l = atomicAdd(&n_runs[bb].y, (unsigned)n_l);
-            at_s = __shfl_sync(FULL, at_s, 0);
-            at_l = __shfl_sync(FULL, at_l, 0);
-            const int64_t b0 = bptr[bb], b1 = bptr[bb + 1];
+            if (one_batch) {
+                __syncthreads();               // the turn before has read its places
+                if (lane == 0) {
+                    s_n[0][warp] = n_s;
+                    s_n[1][warp] = n_l;
+                }
+                __syncthreads();
+                if (threadIdx.x < 2) {         // one thread per counter
+                    unsigned all = 0, at[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        at[i] = all;
+                        all += s_n[threadIdx.x][i];
+                    }
+                    const unsigned place = all ? atomicAdd(threadIdx.x ? &n_runs[bb].y : &n_runs[bb].x, all) : 0u;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) s_n[threadIdx.x][i] = place + at[i];
+                }
+                __syncthreads();
+                at_s = s_n[0][warp];
+                at_l = s_n[1][warp];
+            } else {
+                if (lane == 0 && n_s) at_s = atomicAdd(&n_runs[bb].x, n_s);
+                if (lane == 0 && n_l) at_l = atomicAdd(&n_runs[bb].y, n_l);
+                at_s = __shfl_sync(FULL, at_s, 0);
+                at_l = __shfl_sync(FULL, at_l, 0);
+            }
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                const int64_t s = base + 32 * e + lane;
-                if (ms[e] >> lane & 1u) runs[b0 + at_s + __popc(ms[e] & lanemask_lt())] = (int32_t)s;
-                if (ml[e] >> lane & 1u) {
+                const uint32_t s = base + 32u * e + lane;
+                if (sm[e] >> lane & 1u) runs[b0 + at_s + __popc(sm[e] & lanemask_lt())] = (int32_t)s;
+                at_s += __popc(sm[e]);
+            }
+            if (n_l == 0) continue;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const uint32_t s = base + 32u * e + lane;
+                if (lm[e] >> lane & 1u) {
                     // the run's length: doubling steps, then a binary search (the batch's
                     // pairs are sorted by feature)
-                    int64_t lo = s + BSP_LONG, step = BSP_LONG, hi = lo + step;      // bcol[lo] == j
+                    uint32_t lo = s + BSP_LONG, step = BSP_LONG, hi = lo + step;     // bcol[lo] == j
                     while (hi < b1 && bcol[hi] == j[e]) {
                         lo = hi;
                         step *= 2;
                         hi = lo + step;
                     }
-                    if (hi > b1) hi = b1;
+                    hi = min(hi, b1);
                     while (hi - lo > 1) {
-                        const int64_t mid = lo + ((hi - lo) >> 1);
+                        const uint32_t mid = lo + ((hi - lo) >> 1);
                         if (bcol[mid] == j[e])
                             lo = mid;
                         else
                             hi = mid;
                     }
-                    const int64_t at = b1 - 2 * ((int64_t)at_l + __popc(ml[e] & lanemask_lt()) + 1);
+                    const uint32_t at = b1 - 2 * (at_l + __popc(lm[e] & lanemask_lt()) + 1);
                     runs[at] = (int32_t)s;
                     runs[at + 1] = (int32_t)(lo + 1 - s);
                 }
-                at_s += __popc(ms[e]);
-                at_l += __popc(ml[e]);
+                at_l += __popc(lm[e]);
             }
         }
     }

@@ -129,3 +129,9 @@ def test_many_short_runs(turns):
         p = synthdata.from_arrays(row_ptr, np.arange(n), rng.standard_normal(n).astype(np.float32),
                                   rng.standard_normal(len(row_ptr) - 1), n_cols=n + 3, loss="squared", eta=0.01)
         _equal(p, p.n_rows, epochs=1)
+
+
+@pytest.mark.parametrize("batch", [600_000, 130_000])
+def test_run_lists_of_large_batches(batch):
+    # 12M pairs: the run lists' blocks take several turns, of one batch and of two
+    _equal(synthdata.generate("low-conflict", n_rows=600_000, n_cols=3_000_000, k=20, k_lo=20), batch, epochs=1)
