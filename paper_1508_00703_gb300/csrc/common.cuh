@@ -434,6 +434,7 @@ struct pdb_bsp_plan {
     float *bval;
     int32_t *runs;            // first pairs of each batch's runs (same feature)
     uint2 *n_runs;            // [n_batches] short and long runs
+    pdb::Block arrays;        // holds the device arrays
 };
 
 namespace pdb {

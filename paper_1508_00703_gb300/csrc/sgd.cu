@@ -1120,12 +1120,12 @@ int pdb_bsp_plan_build(const pdb_conflicts *c, int64_t batch, pdb_bsp_plan **out
         p->ev_use = nullptr;
     }
     p->n_batches = N > 0 ? (N + batch - 1) / batch : 0;
-    int rc = alloc((void **)&p->bptr, sizeof(int64_t) * (p->n_batches + 1), s);
-    rc = rc ? rc : alloc((void **)&p->bcol, sizeof(int32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&p->brow, sizeof(int32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&p->bval, sizeof(float) * nnz, s);
-    rc = rc ? rc : alloc((void **)&p->runs, sizeof(int32_t) * nnz, s);
-    rc = rc ? rc : alloc((void **)&p->n_runs, sizeof(uint2) * std::max<int64_t>(p->n_batches, 1), s);
+    int rc = alloc_block(p->arrays, {{(void **)&p->bptr, sizeof(int64_t) * (p->n_batches + 1)},
+                                     {(void **)&p->bcol, sizeof(int32_t) * nnz},
+                                     {(void **)&p->brow, sizeof(int32_t) * nnz},
+                                     {(void **)&p->bval, sizeof(float) * nnz},
+                                     {(void **)&p->runs, sizeof(int32_t) * nnz},
+                                     {(void **)&p->n_runs, sizeof(uint2) * std::max<int64_t>(p->n_batches, 1)}}, s);
     rc = rc ? rc : bsp_sort(cm, c->val, batch, p->n_batches, p->bcol, p->brow, p->bval, p->bptr, p->runs, p->n_runs, s);
     if (rc == PDB_OK && cudaPeekAtLastError() != cudaSuccess) rc = PDB_ECUDA;
     // the host keeps the batches' pair bounds (apply needs them to size its launch)
@@ -1193,8 +1193,7 @@ void pdb_bsp_plan_free(pdb_bsp_plan *p)
         cudaEventDestroy(p->ev_use);
     }
     cudaGetLastError();
-    for (void *q : {(void *)p->bptr, (void *)p->bcol, (void *)p->brow, (void *)p->bval, (void *)p->runs, (void *)p->n_runs})
-        if (q) cudaFreeAsync(q, own_stream());
+    release(p->arrays, own_stream());
     delete[] p->h_bptr;
     delete p;
 }
