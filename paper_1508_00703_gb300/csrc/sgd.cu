@@ -175,6 +175,63 @@ __device__ __forceinline__ bool gather_ready(const unsigned long long *rec, cons
     }
 }
 
+// An example of more ids than a warp's registers hold: wait and gather L elements per
+// lane at a time, then a second pass (this example owns its features until it
+// writes them, so re-reading the records returns the same weights).  Two epochs with
+// one element per lane at a time, each waited for by the whole warp, and with eight:
+// 3000 rows of 500 uniform ids over 60000 features 87.7 and 47.9 ms, 5000 of 1000 over
+// 20M 32.8 and 20.0, 1551 of 293 zipf-like ids over 969 features 23.5 and 20.5.
+template <int L>
+__device__ __forceinline__ bool long_example(int64_t b, int k, float yt, unsigned base, unsigned next_base,
+                                        const int32_t *__restrict__ col, const float *__restrict__ val,
+                                        const uint32_t *__restrict__ gate, unsigned long long *rec, int loss, float eta,
+                                        int *status, uint64_t timeout, uint64_t *trace, int64_t idx)
+{
+    const int lane = threadIdx.x & 31;
+    float acc = 0.0f;
+    for (int i0 = 0; i0 < k; i0 += 32 * L) {
+        int j[L];
+        float x[L], wv[L];
+        unsigned want[L], have = 0;
+#pragma unroll
+        for (int r = 0; r < L; ++r) {
+            const int i = i0 + r * 32 + lane;
+            have |= i < k ? 1u << r : 0u;
+            j[r] = i < k ? col[b + i] : 0;
+            x[r] = i < k ? (val ? val[b + i] : 1.0f) : 0.0f;
+            want[r] = base + (i < k ? gate[b + i] & GATE_RANK : 0u);
+            wv[r] = 0.0f;
+        }
+        if (!gather_ready<L>(rec, j, want, have, wv, status, timeout)) return false;
+#pragma unroll
+        for (int r = 0; r < L; ++r)
+            if (have >> r & 1u) acc = __fmaf_rn(wv[r], x[r], acc);
+    }
+    trace_mark(trace, idx, 0);
+    const float m = warp_combine_latency(acc);
+    const float c = dev_step(loss, m, yt, eta);
+    trace_mark(trace, idx, 1);   // before any write is visible
+    for (int i = lane; i < k; i += 32) {
+        const int jj = col[b + i];
+        const float xx = val ? val[b + i] : 1.0f;
+        const uint32_t g = gate[b + i];
+        const float wo = __uint_as_float((unsigned)ld_rec(rec + jj));
+        st_rec(rec + jj, __fsub_rn(wo, __fmul_rn(c, xx)), (g & GATE_LAST) ? next_base : base + (g & GATE_RANK) + 1u);
+    }
+    return true;
+}
+
+// The widest kernel's, apart from its code: inlined there it slows the shorter rows
+// (20000 rows of 256 ids over 20M features 0.45 -> 0.55 ms).  The narrower kernels
+// meet no such row (they are chosen by the longest one).
+__device__ __noinline__ bool long_example_apart(int64_t b, int k, float yt, unsigned base, unsigned next_base,
+                                                const int32_t *__restrict__ col, const float *__restrict__ val,
+                                                const uint32_t *__restrict__ gate, unsigned long long *rec, int loss,
+                                                float eta, int *status, uint64_t timeout, uint64_t *trace, int64_t idx)
+{
+    return long_example<8>(b, k, yt, base, next_base, col, val, gate, rec, loss, eta, status, timeout, trace, idx);
+}
+
 // one example under the ready protocol; false when a wait gave up
 template <int R>
 __device__ __forceinline__ bool ready_example(int t, unsigned base, unsigned next_base,
@@ -217,30 +274,10 @@ __device__ __forceinline__ bool ready_example(int t, unsigned base, unsigned nex
             if (r * 32 + lane < k) st_rec(rec + j[r], __fsub_rn(wv[r], __fmul_rn(c, x[r])), next[r]);
         return true;
     }
-    // long example: wait and gather element by element, then a second pass
-    // (this example owns its features until it writes them, so re-reading
-    // the records returns the same weights)
-    float acc = 0.0f;
-    for (int i = lane; i - lane < k; i += 32) {
-        const bool in = i < k;
-        const int j1[1] = {in ? col[b + i] : 0};
-        const unsigned w1[1] = {in ? base + (gate[b + i] & GATE_RANK) : 0u};
-        float v1[1] = {0.0f};
-        if (!gather_ready<1>(rec, j1, w1, in ? 1u : 0u, v1, status, timeout)) return false;
-        if (in) acc = __fmaf_rn(v1[0], val ? val[b + i] : 1.0f, acc);
-    }
-    trace_mark(trace, idx, 0);
-    const float m = warp_combine_latency(acc);
-    const float c = dev_step(loss, m, yt, eta);
-    trace_mark(trace, idx, 1);   // before any write is visible
-    for (int i = lane; i < k; i += 32) {
-        const int jj = col[b + i];
-        const float xx = val ? val[b + i] : 1.0f;
-        const uint32_t g = gate[b + i];
-        const float wo = __uint_as_float((unsigned)ld_rec(rec + jj));
-        st_rec(rec + jj, __fsub_rn(wo, __fmul_rn(c, xx)), (g & GATE_LAST) ? next_base : base + (g & GATE_RANK) + 1u);
-    }
-    return true;
+    if constexpr (R < 8)
+        return long_example<1>(b, k, yt, base, next_base, col, val, gate, rec, loss, eta, status, timeout, trace, idx);
+    else
+        return long_example_apart(b, k, yt, base, next_base, col, val, gate, rec, loss, eta, status, timeout, trace, idx);
 }
 
 template <int R>

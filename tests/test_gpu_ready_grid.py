@@ -56,3 +56,10 @@ def test_many_epochs_of_few_examples(n):
 def test_tickets_and_grids(chunk, blocks):
     _equal(synthdata.generate("tiny", n_rows=3000, n_cols=COLS, k=20, k_lo=3, epochs=2, seed=4),
            dict(ticket_chunk=chunk, blocks_per_sm=blocks))
+
+
+@pytest.mark.parametrize("k", [511, 512, 513, 768, 769, 1030])
+def test_long_rows(k):
+    # rows of several times the ids a warp takes at once (256), with shorter ones among them
+    for lo in (k, 0):
+        _equal(synthdata.generate("tiny", n_rows=200, n_cols=COLS, k=k, k_lo=lo, ids="zipf", zipf_s=1.0, epochs=2, seed=k))
