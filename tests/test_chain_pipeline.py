@@ -1,59 +1,74 @@
 """A model of the CHAIN engine's pipeline schedule, on the CPU.
 
 One thread block runs the examples in data order, G per pipeline step, and
-its warps work on different steps in the same iteration of the step loop,
+its warps work on different steps in the same iteration t of the step loop,
 separated only by the __syncthreads that ends each iteration:
 
-  W   (G / 2 warps, two examples each)  writes through the new weights of
-                   step t - 1 whose next occurrence is not pushed; the first
-                   also copies row bounds L = DS + BS + 1 steps ahead into a
-                   ring of RP;
-  A   (one warp per example of a step)  copies ids, link words and values of
-                   step t + DS into the example's slot of a ring of SLOTS;
-  B   (the same warps)  gathers, for step t + BS, the weights nobody pushes
-                   from global w, and where each new weight will be stored;
-  C   (the compute warp)  runs the examples of step t in order, each reading
-                   its weights from its slot and storing each new weight
-                   into the next occurrence's slot when that lies within
-                   D = G * DS examples (a push), else into its own output
-                   slot for W.
-
-The asynchronous copies (row bounds, ids, link words, values, labels,
-gathered weights) of one iteration land by the end of iteration + INFLIGHT:
-until then the model counts their source and destination cells as touched by
-the copying warp in every iteration they may still be moving.
-
-C comes in two forms.  For rows of more than 32 ids, every example but the
-first of a step fetches its weights while the example before it is still
-computing, before that example's stores; a weight whose previous occurrence
-is that very example is taken from it directly.  For rows of up to 32 ids,
-every example -- the first of a step too, then during the last example of
-the step before -- is fetched while the example before it computes, after
-the stores of the example before that; the stores of an example wait for the
-next example's margin to start, and the last example of a step stores before
-the step's barrier.
+  P   (G warps, example g of a step each)  keeps its loads in registers from
+                   one iteration to the next: row bounds of step t + RS, with
+                   those of the iteration before the ids, link words, values
+                   and label of step t + AS, with those the global weights
+                   nobody pushes of step t + BS; writes step t + BS's values,
+                   label and store addresses (ring of XS example slots) and
+                   write-through ids (ring of WS), and the weights gathered
+                   one iteration ago, for step t + BS - 1, to the weight slots
+                   (ring of WS);
+  C   (one warp)  runs the examples of step t in order, each reading its
+                   weights, label, values and store addresses from its slots
+                   and storing each new weight to its address: the slot of the
+                   feature's next occurrence when that lies within D = G * DS
+                   examples (a push), its own out slot (ring of OS) otherwise.
+                   Values are read one example ahead, so the last example of a
+                   step reads those of the next step's first.  When a margin
+                   lies outside the fast derivative's range the whole step runs
+                   again;
+  W   (G / WPER warps)  writes step t - 1's out slots through to global w.
 
 The model replays that schedule with the link words the engine builds from
-the conflict chains (including the mark of a previous occurrence in the
-example just before) and checks, on problems full of near repeats: every
+the conflict chains and checks, on problems full of near repeats: every
 example uses, for every feature, exactly the weight its previous occurrence
-wrote (in the epoch, or the last one of the epoch before); global w ends each
-epoch holding each feature's last writer; no two warps touch one shared or
-global cell in the same iteration unless both only read it; every row bound
-read comes from the ring entry of that very example; every slot the compute
-warp reads holds the example it reads it for.  The same checks fail when the
-constants break the engine's compile-time conditions (a gather one step
-earlier, a shorter forwarding window, a ring of 16 slots, copies left in
-flight one step longer)."""
+wrote (in the epoch, or the last one of the epoch before), also in steps that
+run twice; every slot the compute warp reads holds the example it reads it for;
+global w ends each epoch holding each feature's last writer; no two warps touch
+one shared or global cell in the same iteration unless both only read it.  A
+gathered weight's load may complete one iteration after its issue: its global
+cell counts as read in both.
+
+The rings and distances are read from the engine's source, so a change there is
+checked here.  The same checks fail when a constant breaks one of the engine's
+compile-time conditions (each ring one power of two shorter, a shorter and a
+longer forwarding window, weights stored in the step that reads them), when a
+repeated step is not run again whole, and when values are read a step instead of
+an example ahead."""
+import os
+import re
+
 import numpy as np
 import pytest
 
 import oracle
 import synthdata
 
-# the engine's pipeline shapes: rows of up to 128 ids, and of up to 256
-ENGINE = dict(G=8, DS=5, BS=3, SLOTS=64, RP=128, INFLIGHT=1)
-ENGINE_LONG = dict(G=4, DS=5, BS=3, SLOTS=32, RP=128, INFLIGHT=1)
+SRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1508_00703_gb300", "csrc", "chain.cu")
+
+
+def _engine():
+    """The constants of ChainCfg, the same for every row width."""
+    body = re.search(r"struct ChainCfg \{(.*?)\};", open(SRC).read(), re.S).group(1)
+    c = {}
+    for decl in re.findall(r"static constexpr int ([^;]*);", body):
+        for item in decl.split(","):
+            name, expr = item.split("=")
+            if "R" not in re.findall(r"\w+", expr):              # all but the longest row
+                c[name.strip()] = eval(expr, {}, c)
+    return {k: c[k] for k in ("G", "DS", "BS", "AS", "RS", "PS", "D", "XS", "WS", "OS", "WPER")}
+
+
+ENGINE = _engine()
+
+
+def test_constants_were_found():
+    assert ENGINE["D"] == ENGINE["G"] * ENGINE["DS"] and ENGINE["AS"] == ENGINE["BS"] + 1 and ENGINE["RS"] == ENGINE["AS"] + 1
 
 
 def _links(p, D):
@@ -61,17 +76,14 @@ def _links(p, D):
     prev, nxt = ch["prev"], ch["next"]
     row_of = np.repeat(np.arange(p.n_rows), np.diff(p.row_ptr))
     recv = np.zeros(p.nnz, bool)
-    late = np.zeros(p.nnz, bool)
     push = {}
     for q in range(p.nnz):
         t = row_of[q]
         if prev[q] >= 0 and t - row_of[prev[q]] <= D:
             recv[q] = True
-        if prev[q] >= 0 and row_of[prev[q]] == t - 1:
-            late[q] = True
         if nxt[q] >= 0 and row_of[nxt[q]] - t <= D:
             push[q] = (int(row_of[nxt[q]] - t), int(nxt[q] - p.row_ptr[row_of[nxt[q]]]))
-    return recv, push, late
+    return recv, push
 
 
 class _Iteration:
@@ -92,189 +104,139 @@ class _Iteration:
             assert len(others) == 1, ("two warps touch one cell in one iteration", t, cell, sorted(others))
 
 
-def _simulate(p, epochs, G, DS, BS, SLOTS, RP, INFLIGHT, D=None, one_per_lane=True):
-    D = G * DS if D is None else D
-    L = DS + BS + 1
-    N = p.n_rows
-    rp = p.row_ptr
-    recv, push, late = _links(p, D)
+def _simulate(p, epochs, G, DS, BS, AS, RS, PS, D, XS, WS, OS, WPER, twice=(), redo="whole", ahead=True):
+    """twice: examples whose step runs again; redo: "whole" step, or (planted) that example alone; ahead:
+    values read one example ahead (planted: a whole step ahead)."""
+    N, rp = p.n_rows, p.row_ptr
+    K = max(1, int(np.max(np.diff(rp))) if N else 1)      # slots are written to their full width
+    recv, push = _links(p, D)
     steps = (N + G - 1) // G
-    slot_of = lambda r: r & (SLOTS - 1)
-    # weights are tracked as the example (epoch, id) that wrote them; None = w0
-    w = {}
-    last_writer = {}                      # feature -> (epoch, example) of its latest write in data order
+    mem = {}                              # shared memory: cell -> what it holds
+    w = {}                                # global: feature -> (epoch, example) of its writer, None = w0
+    last_writer = {}
     for ep in range(epochs):
-        ring = {}                         # rp ring: index -> example whose bound it holds
-        col, wp, out, pa, xa, kk, ys = {}, {}, {}, {}, {}, {}, {}
-        tables = dict(rp=ring, col=col, xa=xa, y=ys, wp=wp)
-        inflight = []                     # asynchronous copies: (last iteration, warp, cells, effects)
-
-        def bounds(it, warp, r):
-            if r < 0 or r >= N:
-                return None
-            for e in (r, r + 1):
-                it.r(warp, ("rp", e & (RP - 1)))
-                assert ring.get(e & (RP - 1)) == e, ("row bound not in the ring", r, e)
-            return int(rp[r]), int(rp[r + 1] - rp[r])
-
         expect = dict(last_writer)        # the weight the next occurrence of each feature must read
-        for t in range(-L, steps + 1):
+        bounds, loaded, gathered = {}, {}, {}     # registers of warp P g
+        late = []                         # global cells of loads that may complete in the next iteration
+        vals = None                       # C's registers: the values of the next example
+        for t in range(-PS, steps + 1):
             it = _Iteration()
-            effects = []                  # plain stores: land at the end of this iteration
-            copies = {}                   # warp -> (cells read, cells written, effects) of this iteration's copies
+            effects = []                  # stores: visible to the others after the iteration's barrier
+            for warp, cell in late:
+                it.r(warp, cell)
+            late = []
 
-            def copy(warp, src, dst, key, v):
-                c = copies.setdefault(warp, ([], [], []))
-                if src is not None:
-                    c[0].append(src)
-                c[1].append(dst)
-                c[2].append((key, v))
+            def store(warp, cell, v):
+                it.w(warp, cell)
+                effects.append((cell, v))
 
-            # W: warp i writes examples 2i, 2i + 1 of step t - 1; W0 also copies row bounds
-            for warp, gs in ((f"W{i}", range(2 * i, 2 * i + 2)) for i in range(G // 2)):
-                for g in gs:
-                    r = (t - 1) * G + g
-                    bk = bounds(it, warp, r)
-                    if bk is None:
-                        continue
-                    b, k = bk
-                    s = slot_of(r)
-                    for i in range(k):
-                        it.r(warp, ("link", s, i))
-                        if b + i not in push:
-                            it.r(warp, ("col", s, i))
-                            it.r(warp, ("out", s, i))
-                            j = col[(s, i)]
-                            it.w(warp, ("w", j))
-                            effects.append(("w", j, out[(s, i)]))
-            for lane in range(G):
-                e = (t + L) * G + lane
-                if 0 <= e <= N:
-                    copy("W0", ("row_ptr", e), ("rp", e & (RP - 1)), ("rp", e & (RP - 1)), e)
-            # A and B: one warp per example g of a step
             for g in range(G):
-                warp = f"AB{g}"
-                r = (t + DS) * G + g
-                bk = bounds(it, warp, r)
-                if bk is not None:
-                    b, k = bk
-                    s = slot_of(r)
-                    for i in range(k):
-                        copy(warp, None, ("col", s, i), ("col", (s, i)), int(p.col[b + i]))
-                        copy(warp, None, ("link", s, i), ("link", (s, i)), None)
-                        copy(warp, None, ("xa", s, i), ("xa", (s, i)), (r, i))
-                    copy(warp, None, ("y", s), ("y", s), r)
+                warp = f"P{g}"
+                # the weights gathered one iteration ago, to step t + BS - 1's slots
+                for r, i, v in gathered.pop(g, []):
+                    store(warp, ("wp", r % WS, i), v)
+                # step t + BS, from the ids and link words loaded one iteration ago
                 r = (t + BS) * G + g
-                bk = bounds(it, warp, r)
-                if bk is not None:
-                    b, k = bk
-                    s = slot_of(r)
-                    for i in range(k):
-                        it.r(warp, ("link", s, i))
-                        it.r(warp, ("col", s, i))
-                        if not recv[b + i]:
-                            j = col.get((s, i))
-                            assert j == int(p.col[b + i]), ("gather before the id landed", r, i)
-                            copy(warp, ("w", j), ("wp", s, i), ("wp", (s, i)), w.get(j))
-                        it.w(warp, ("pa", s, i))
-                        if b + i in push:
-                            dr, e = push[b + i]
-                            effects.append(("pa", (s, i), ("wp", slot_of(r + dr), e)))
+                if 0 <= r < N:
+                    assert loaded[g] == r, ("registers of another example", r, loaded[g])
+                    b, k = int(rp[r]), int(rp[r + 1] - rp[r])
+                    new = []
+                    for i in range(K):
+                        q, inside = b + i, i < k
+                        if inside and not recv[q]:
+                            j = int(p.col[q])
+                            it.r(warp, ("w", j))
+                            late.append((warp, ("w", j)))
+                            new.append((r, i, w.get(j)))
+                        elif not inside:
+                            new.append((r, i, "zero"))
+                        if inside and q in push:
+                            dr, e = push[q]
+                            to = ("wp", (r + dr) % WS, e)
                         else:
-                            effects.append(("pa", (s, i), ("out", s, i)))
-                    it.w(warp, ("kk", s))
-                    effects.append(("kk", s, r))
-            for warp, (rd, wr, eff) in copies.items():
-                inflight.append((t + INFLIGHT, warp, rd, wr, eff))
-            # copies still moving touch their cells in every iteration until they land
-            for last, warp, rd, wr, _ in inflight:
-                for cell in rd:
-                    it.r(warp, cell)
-                for cell in wr:
-                    it.w(warp, cell)
-            # C: the compute warp, examples of step t in data order (its own
-            # accesses are ordered; its stores are visible to its later reads)
+                            to = ("out", r % OS, i) if inside else None
+                        store(warp, ("pa", r % XS, i), (r, to))
+                        store(warp, ("wcol", r % WS, i), (r, int(p.col[q]) if inside and q not in push else -1))
+                        store(warp, ("xa", r % XS, i), (r, i) if inside else (r, "-0"))
+                    store(warp, ("y", r % XS), r)
+                    gathered[g] = new
+                r = (t + AS) * G + g
+                if 0 <= r < N:
+                    assert bounds[g] == r, ("row bounds of another example", r, bounds[g])
+                    loaded[g] = r
+                r = (t + RS) * G + g
+                if 0 <= r < N:
+                    bounds[g] = r
+            for i in range(G // WPER):
+                for r in range((t - 1) * G + i * WPER, (t - 1) * G + (i + 1) * WPER):
+                    if not (t >= 1 and r < N):
+                        continue
+                    for e in range(K):
+                        it.r(f"W{i}", ("wcol", r % WS, e))
+                        it.r(f"W{i}", ("out", r % OS, e))
+                        of, j = mem[("wcol", r % WS, e)]
+                        assert of == r, ("write-through ids of another example", r, of)
+                        if j >= 0:
+                            store(f"W{i}", ("w", j), mem[("out", r % OS, e)])
             if 0 <= t < steps:
-                local = {}
+                local = {}                # C's own stores, visible to its later reads
 
-                def fetch(r):
-                    # the slot's length, label, values, ids, store words and weights
+                def read(cell):
+                    it.r("C", cell)
+                    return local.get(cell, mem.get(cell))
+
+                def load_values(r):
+                    return [read(("xa", r % XS, i)) for i in range(K)]
+
+                def run(r, bad):
+                    """One example; bad: in a first run of its step that gives wrong weights from here on."""
+                    nonlocal vals
                     b, k = int(rp[r]), int(rp[r + 1] - rp[r])
-                    s = slot_of(r)
-                    it.r("C", ("kk", s))
-                    it.r("C", ("y", s))
-                    assert kk.get(s) == r and ys.get(s) == r, ("slot holds another example", r, kk.get(s), ys.get(s))
-                    got, targets = [], []
-                    for i in range(k):
-                        for arr in ("xa", "pa", "wp"):
-                            it.r("C", (arr, s, i))
-                        assert xa.get((s, i)) == (r, i), ("value of another example", r, i, xa.get((s, i)))
-                        assert col[(s, i)] == int(p.col[b + i]), ("id of another example", r, i)
-                        got.append(local.get(("wp", s, i), wp.get((s, i))))
-                        targets.append(pa[(s, i)])
-                    return got, targets
-
-                def compute(r, got, from_before):
-                    # the weights the margin uses: a late one from the example just before
-                    b, k = int(rp[r]), int(rp[r + 1] - rp[r])
-                    for i in range(k):
-                        j = int(p.col[b + i])
-                        v = (ep, r - 1) if from_before and late[b + i] else got[i]
-                        assert v == expect.get(j), ("wrong weight read", ep, r, j, v, expect.get(j))
-                    for i in range(k):
-                        expect[int(p.col[b + i])] = (ep, r)
-
-                def store(r, targets):
-                    for target in targets:
-                        it.w("C", target)
-                        local[target] = (ep, r)
+                    got = [read(("wp", r % WS, i)) for i in range(K)]
+                    x = vals
+                    assert read(("y", r % XS)) == r
+                    vals = load_values(r + (1 if ahead else G))
+                    assert x == [(r, i) if i < k else (r, "-0") for i in range(K)], ("values of another example", r, x)
+                    assert all(v == "zero" for v in got[k:]), ("padding reads a weight", r, got)
+                    if not bad:
+                        for i in range(k):
+                            j = int(p.col[b + i])
+                            assert got[i] == expect.get(j), ("wrong weight read", ep, r, j, got[i], expect.get(j))
+                    for i in range(K):
+                        of, to = read(("pa", r % XS, i))
+                        assert of == r, ("store address of another example", r, of)
+                        if to is not None:
+                            it.w("C", to)
+                            local[to] = ("bad", ep, r) if bad else (ep, r)
+                    if not bad:
+                        for i in range(k):
+                            expect[int(p.col[b + i])] = (ep, r)
 
                 r0, r1 = t * G, min(N, t * G + G)
-                if one_per_lane:
-                    if t == 0:
-                        nxt = fetch(0)
+                flagged = [r for r in range(r0, r1) if (ep, r) in twice]
+                if t == 0:
+                    vals = load_values(0)
+                if not flagged:
                     for r in range(r0, r1):
-                        cur = nxt
-                        if r > r0:
-                            store(r - 1, prev_targets)
-                        if r + 1 < N:
-                            nxt = fetch(r + 1)
-                        compute(r, cur[0], True)
-                        prev_targets = cur[1]
-                    store(r1 - 1, prev_targets)
+                        run(r, False)
                 else:
-                    nxt = fetch(r0)
-                    for g, r in enumerate(range(r0, r1)):
-                        cur = nxt
-                        if r + 1 < r1:
-                            nxt = fetch(r + 1)        # before this example's stores
-                        compute(r, cur[0], g > 0)
-                        store(r, cur[1])
-                effects.extend(("cstore", cell, v) for cell, v in local.items())
+                    before = dict(expect)
+                    for r in range(r0, r1):              # from the first flagged example on, wrong
+                        run(r, r >= flagged[0])
+                    expect = before
+                    again = range(r0, r1) if redo == "whole" else flagged
+                    vals = load_values(again[0])
+                    for r in again:
+                        run(r, False)
+                effects.extend(local.items())
             it.check(t)
-            # the iteration's plain stores land before the next iteration
-            # (__syncthreads), and so do the copies whose last iteration it is
-            landed = [e for last, _, _, _, eff in inflight if last == t for e in eff]
-            inflight = [c for c in inflight if c[0] > t]
-            for kind, key, v in effects + [(k, key, v) for (k, key), v in landed]:
-                if kind == "w":
-                    w[key] = v
-                elif kind in tables:
-                    tables[kind][key] = v
-                elif kind == "link":
-                    pass
-                elif kind == "kk":
-                    kk[key] = v
-                elif kind == "pa":
-                    pa[key] = v
+            for cell, v in effects:
+                if cell[0] == "w":
+                    w[cell[1]] = v
                 else:
-                    if key[0] == "wp":
-                        wp[(key[1], key[2])] = v
-                    else:
-                        out[(key[1], key[2])] = v
+                    mem[cell] = v
         last_writer = expect
-        # the drain at the end of the epoch leaves every feature's last writer in w
-        for j, v in last_writer.items():
+        for j, v in last_writer.items():                  # the drain leaves every feature's last writer in w
             assert w.get(j) == v, ("w after the epoch", ep, j, w.get(j), v)
 
 
@@ -283,138 +245,93 @@ def _problem(seed, rng):
                               k=int(rng.integers(1, 6)), k_lo=0, ids="zipf" if seed % 2 else "uniform", zipf_s=1.2)
 
 
-FORMS = [(ENGINE, True), (ENGINE, False), (ENGINE_LONG, False)]     # (shape, one element per lane)
+def _periods(n=150):
+    """A feature for every distance from 28 to 72 between its occurrences (the window and the rings end in there)."""
+    ds = range(28, 73)
+    rows = [[d - 28 for d in ds if (t + d // 2) % d == 0] for t in range(n)]
+    return synthdata.from_arrays(np.r_[0, np.cumsum([len(r) for r in rows])], np.concatenate(rows).astype(np.int32), None,
+                                 np.ones(n), n_cols=len(ds))
 
 
-@pytest.mark.parametrize("cfg,one_per_lane", FORMS)
-@pytest.mark.parametrize("seed", range(8))
-def test_chain_pipeline_schedule(seed, cfg, one_per_lane):
+def test_chain_pipeline_every_distance():
+    p = _periods()
+    _simulate(p, epochs=2, **ENGINE)
+    _simulate(p, epochs=2, twice={(0, r) for r in range(0, p.n_rows, 5)}, **ENGINE)
+
+
+@pytest.mark.parametrize("seed", range(10))
+def test_chain_pipeline_schedule(seed):
     rng = np.random.default_rng(700 + seed)
-    _simulate(_problem(seed, rng), epochs=2, one_per_lane=one_per_lane, **cfg)
+    p = _problem(seed, rng)
+    _simulate(p, epochs=2, **ENGINE)
+    # and with steps that run again: a tenth of the examples outside the fast derivative's range
+    twice = {(ep, r) for ep in range(2) for r in range(p.n_rows) if rng.random() < 0.1}
+    _simulate(p, epochs=2, twice=twice, **ENGINE)
 
 
-@pytest.mark.parametrize("cfg,one_per_lane", FORMS)
-def test_chain_pipeline_one_feature_and_ragged(cfg, one_per_lane):
+def test_chain_pipeline_one_feature_and_ragged():
     # every example holds feature 0: every weight is pushed; and a ragged
     # problem with empty examples and a short last step
     n = 37
     p = synthdata.from_arrays(np.arange(n + 1), np.zeros(n, np.int32), None, np.ones(n), n_cols=1)
-    _simulate(p, epochs=3, one_per_lane=one_per_lane, **cfg)
+    _simulate(p, epochs=3, **ENGINE)
     q = synthdata.generate("tiny", seed=5, n_rows=101, n_cols=7, k=4, k_lo=0)
-    _simulate(q, epochs=2, one_per_lane=one_per_lane, **cfg)
+    _simulate(q, epochs=2, twice={(1, 0), (1, 100), (0, 50)}, **ENGINE)
 
 
-@pytest.mark.parametrize("change", [dict(BS=2), dict(D=32), dict(SLOTS=32), dict(INFLIGHT=2)])
-def test_chain_pipeline_model_rejects_broken_constants(change):
-    cfg, change = dict(ENGINE), dict(change)
-    D = change.pop("D", None)
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 15, 16, 17, 40, 41, 63, 65])
+def test_chain_pipeline_short_data(n):
+    for k in (1, 3):
+        p = synthdata.generate("tiny", seed=n, n_rows=n, n_cols=5, k=k, k_lo=k)
+        _simulate(p, epochs=3, twice={(1, n - 1)}, **ENGINE)
+
+
+def _fails(change, **plant):
+    cfg = dict(ENGINE)
     cfg.update(change)
     failures = 0
-    for seed in range(4):
+    for seed in range(6):
         rng = np.random.default_rng(800 + seed)
+        p = _problem(seed, rng) if seed else _periods()
+        twice = {(0, r) for r in range(p.n_rows) if rng.random() < 0.1}
         try:
-            _simulate(_problem(seed, rng), epochs=2, D=D, **cfg)
+            _simulate(p, epochs=2, twice=twice, **plant, **cfg)
         except AssertionError:
             failures += 1
-    assert failures > 0
+    return failures
 
 
-def _handoff_program(P, N, G, epochs):
-    """The operations compute warp P (0: even examples, 1: odd ones) issues,
-    in the kernel's order, for rows of up to 32 ids: waits on and arrivals at
-    the named barriers C (c published) and S (stores done) of each warp, and
-    the block-wide barrier that ends each step."""
-    steps = (N + G - 1) // G
-    for ep in range(epochs):
-        for t in range(steps):
-            r0, r1 = t * G, min(N, t * G + G)
-            for r in range(r0 + P, r1, 2):
-                if r > 0:
-                    yield ("wait", ("C", P ^ 1), (ep, r))
-                yield ("use", "c", (ep, r))           # reads c of r - 1, computes c of r
-                if r > 0:
-                    yield ("wait", ("S", P ^ 1), (ep, r))
-                if r + 1 < N:
-                    yield ("arrive", ("C", P), (ep, r))
-                yield ("use", "store", (ep, r))
-                if r + 1 < N:
-                    yield ("arrive", ("S", P), (ep, r))
-            yield ("block", None, (ep, t))
+def _at_distance(BS):
+    return dict(BS=BS, AS=BS + 1, RS=BS + 2)
 
 
-def _run_handoffs(N, G, epochs, seed):
-    rng = np.random.default_rng(seed)
-    progs = [_handoff_program(P, N, G, epochs) for P in (0, 1)]
-    nxt = [next(p, None) for p in progs]
-    bars = {}                    # barrier -> (warp that arrived or waits, op kind, example)
-    waiting = [None, None]       # a warp blocked in a wait
-    block = [None, None]         # a warp at the block barrier: its (epoch, step)
-    computed, stored, released = set(), set(), {}
-    while nxt[0] is not None or nxt[1] is not None or any(waiting):
-        ready = [P for P in (0, 1) if nxt[P] is not None and waiting[P] is None and block[P] is None]
-        if not ready:
-            # only the block barrier can release now: both warps (or the one with work left) must be there
-            live = [P for P in (0, 1) if block[P] is not None]
-            assert live and not any(waiting), ("deadlock", N, G, nxt, waiting, block, bars)
-            assert all(block[P] == block[live[0]] for P in live)
-            for P in live:
-                block[P] = None
-                nxt[P] = next(progs[P], None)
-            continue
-        P = int(rng.choice(ready))
-        kind, bar, ex = nxt[P]
-        if kind == "block":
-            block[P] = ex
-            other = P ^ 1
-            if nxt[other] is None or block[other] is not None:
-                for Q in (0, 1):
-                    if block[Q] is not None:
-                        block[Q] = None
-                        nxt[Q] = next(progs[Q], None)
-            continue
-        if kind == "use":
-            ep, r = ex
-            if bar == "c":
-                # the weights of r's late elements come from r - 1, which must have published c
-                assert r == 0 or (ep, r - 1) in released.get(("C", P ^ 1), set()), ("c of r - 1 not published", ex)
-                computed.add(ex)
-            else:
-                stored.add(ex)
-        elif kind == "arrive":
-            held = bars.get(bar)
-            assert held is None or held[1] == "wait", ("two arrivals before a wait", bar, held, ex)
-            assert bar[1] == P
-            if held is None:
-                bars[bar] = (P, "arrive", ex)
-            else:
-                # the waiting warp is released; it waited for exactly this example
-                W = held[0]
-                assert W == P ^ 1 and held[2][1] == ex[1] + 1, ("wrong pairing", bar, held, ex)
-                released.setdefault(bar, set()).add(ex)
-                del bars[bar]
-                waiting[W] = None
-                nxt[W] = next(progs[W], None)
-            if bar[0] == "S":
-                assert ex in stored, ("stores announced before they are issued", ex)
-        elif kind == "wait":
-            held = bars.get(bar)
-            assert bar[1] == P ^ 1
-            if held is None:
-                bars[bar] = (P, "wait", ex)
-                waiting[P] = bar
-                continue
-            assert held[1] == "arrive" and held[2][1] == ex[1] - 1, ("wrong pairing", bar, held, ex)
-            released.setdefault(bar, set()).add(held[2])
-            del bars[bar]
-        nxt[P] = next(progs[P], None)
-    assert not bars, ("a barrier left half used", bars)
-    assert len(computed) == N * epochs and len(stored) == N * epochs
+@pytest.mark.parametrize("change", [
+    dict(XS=ENGINE["XS"] // 2),                       # XS >= (BS + 1) G
+    dict(WS=ENGINE["WS"] // 2),                       # WS >= (DS + 1) G and (BS + 2) G
+    dict(DS=ENGINE["WS"] // ENGINE["G"], D=ENGINE["WS"]),   # the same: a push to its own example's slot, read again
+    dict(OS=ENGINE["OS"] // 2),                       # OS >= 2 G
+    dict(D=(ENGINE["BS"] + 2) * ENGINE["G"] - 2),     # (D + 1) / G >= BS + 2
+    dict(DS=2, D=2 * ENGINE["G"]),
+    _at_distance(1),                                  # BS >= 2
+    _at_distance(4),                                  # values live longer than XS; weights gathered too early
+])
+def test_chain_pipeline_model_rejects_broken_constants(change):
+    assert _fails(change) > 0
 
 
-@pytest.mark.parametrize("N", [0, 1, 2, 3, 7, 8, 9, 15, 16, 17, 40, 63])
-def test_compute_warp_handoffs(N):
-    # the two compute warps' named-barrier protocol: every barrier completes
-    # with one arrival and one wait, for the example just before, in any
-    # interleaving, and nothing is left half used at the end of an epoch
-    for seed in range(30):
-        _run_handoffs(N, G=8, epochs=2, seed=seed)
+@pytest.mark.parametrize("plant", [dict(redo="one"), dict(ahead=False)])
+def test_chain_pipeline_model_rejects_planted_mistakes(plant):
+    assert _fails({}, **plant) > 0
+
+
+def test_element_layout():
+    # rows of up to 64 ids: element i of each 32 at chain_at(i), so that a lane's four neighbouring words hold the
+    # partial sums p, p + 8, p + 16, p + 24 of the margin and its own element is one of them
+    at = [(i & ~31) | ((i & 7) << 2) | ((i >> 3) & 3) for i in range(64)]
+    assert re.search(r"return QUAD<R> \? \(i & ~31\) \| \(\(i & 7\) << 2\) \| \(\(i >> 3\) & 3\) : i;", open(SRC).read())
+    assert sorted(at) == list(range(64))
+    where = {a: i for i, a in enumerate(at)}
+    for lane in range(32):
+        four = [where[(lane & 7) * 4 + e] for e in range(4)]
+        assert four == [lane % 8 + 8 * e for e in range(4)]
+        assert where[(lane & 7) * 4 + (lane >> 3)] == lane
