@@ -1,6 +1,7 @@
 """The conflict build where its passes change form: sizes around a sort tile
-(4096 pairs), around the steps of the scan's chunk length and its two scan
-forms, and around the sizes at which the gate words are brought to position
+(4096 pairs), around the steps of the scan's chunk length, on both sides of the
+switch from the scan inside its last kernel to the one with a kernel of its own
+(128 chunks of 256 tiles), and around the sizes at which the gate words are brought to position
 order by direct stores, by one radix pass over 2^15-slot blocks and by two over
 2^14 (2^22, 2^24, 2^25 positions).  Checked against the definitions on the
 device: csc_pos a stable sort of the ids, feat_ptr its bounds, prev, next and
@@ -24,7 +25,7 @@ def _cuda():
 
 @pytest.mark.parametrize("n", [1, T - 1, T, T + 1, 16 * T, 16 * T + 1, 17 * T, 512 * T, 512 * T + 1, (1 << 22) - 1, 1 << 22,
                                (1 << 22) + 1, 2048 * T, 2048 * T + 3, 1 << 24, (1 << 24) + 1, 1 << 25, (1 << 25) + 5,
-                               16384 * T + 1])
+                               16384 * T + 1, 32768 * T, 32768 * T + 1])
 @pytest.mark.parametrize("cols", [300, 5_000_000])
 def test_build(n, cols):
     g = torch.Generator(device="cuda").manual_seed(n + cols)
