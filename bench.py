@@ -262,6 +262,22 @@ def training_loss(p, X, y, w, torch):
     return float(torch.clamp(1.0 - yy * m, min=0.0).mean())
 
 
+def sgd_kernel(p, mode, optin_smem):
+    """The kernel that ran: the schedule's mode (-1 BSP, -2 admissible delay) and, where a mode has several
+    engines, the library's rule for them (csrc/sgd.cu, csrc/build.cu)."""
+    import numpy as np
+    if mode == 1:          # READY: one block when its shared memory holds every record
+        longest = int(np.diff(p.row_ptr).max()) if p.n_rows else 0
+        block = longest <= 64 and 1 <= p.n_cols and p.n_cols * 8 + 1024 <= optin_smem
+        return "k_sgd_block_ready" if block and p.epochs * p.n_rows < 2 ** 31 - 1024 else "k_sgd_ready"
+    if mode == 2:          # CHAIN: weights in registers for dense rows, in shared memory for rows over 256 ids
+        longest = int(np.diff(p.row_ptr).max()) if p.n_rows else 0
+        dense = (p.nnz == p.n_rows * p.n_cols and longest == p.n_cols <= 1024
+                 and bool(np.all(p.col.reshape(p.n_rows, -1) == np.arange(p.n_cols))))
+        return "k_sgd_dense" if dense else "k_sgd_resident" if longest > 256 else "k_sgd_chain"
+    return {0: "k_sgd_levels", 4: "k_sgd_window", -1: "k_bsp_apply", -2: "k_sgd_ssp"}[mode]
+
+
 def workload_config(name, problem, mode):
     import synthdata
     spec = synthdata.WORKLOADS[name]
@@ -360,8 +376,8 @@ def run_ours(args, rank, world, local_rank):
     resolved = int(phases[0]["sched_mode"])
     if args.delay is not None:
         resolved = -2
-    kname = {pdb.PDB_SCHED_READY: "k_sgd_ready", pdb.PDB_SCHED_LEVELS: "k_sgd_levels", -1: "k_bsp_apply", -2: "k_sgd_ssp",
-             pdb.PDB_SCHED_CHAIN: "k_sgd_chain", pdb.PDB_SCHED_WINDOW: "k_sgd_window"}[resolved]
+    optin = getattr(torch.cuda.get_device_properties(local_rank), "shared_memory_per_block_optin", 232448)
+    kname = sgd_kernel(p, resolved, optin)
     roofline = {"kernel": kname,
                 "bound": "hbm", "achieved": round(sgd_gbs, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(sgd_gbs / peak, 4), "traffic": recorded_traffic(kname, args.workload, p.nnz),
@@ -385,7 +401,7 @@ def run_ours(args, rank, world, local_rank):
                                        {0: "levels", 1: "ready", 2: "chain", 4: "window"}[resolved]
                                        + (" (auto)" if args.mode == "auto" else "")),
                        parallelism=f"replicas{world}" if world > 1 else "single GPU",
-                       ticket_chunk=args.ticket_chunk or 2),
+                       ticket_chunk=args.ticket_chunk or ("default" if resolved == pdb.PDB_SCHED_READY else 2)),
         "roofline": roofline,
         "phases_ms": ({"build_conflicts": ms_build, "bsp_all_epochs": ms_sgd} if batch else
                       {"build_conflicts": ms_build, "schedule": ms_sched, "sgd_all_epochs": ms_sgd,

@@ -106,3 +106,20 @@ def test_recorded_traffic_only_while_the_sources_match(tmp_path, monkeypatch):
     (csrc / "window.cu").write_text("kernel B\n")
     assert bench.recorded_traffic("k_sgd_window", "low-conflict", 1000) is None
     assert bench.recorded_traffic("k_sgd_window", "zipf-1m", 1000) is None
+
+
+def test_roofline_names_the_kernel_that_ran():
+    sys.path.insert(0, ROOT)
+    import bench
+    import synthdata
+    smem = 232448
+    tiny = synthdata.generate("tiny", n_rows=50)
+    assert bench.sgd_kernel(tiny, 1, smem) == "k_sgd_block_ready"
+    assert bench.sgd_kernel(synthdata.generate("tiny", n_rows=50, n_cols=40000), 1, smem) == "k_sgd_ready"
+    assert bench.sgd_kernel(synthdata.generate("tiny", n_rows=50, k=65), 1, smem) == "k_sgd_ready"
+    assert bench.sgd_kernel(tiny, 2, smem) == "k_sgd_chain"
+    assert bench.sgd_kernel(synthdata.generate("tiny", n_rows=50, k=300), 2, smem) == "k_sgd_resident"
+    assert bench.sgd_kernel(synthdata.generate("dense-lr", n_rows=20), 2, smem) == "k_sgd_dense"
+    assert bench.sgd_kernel(synthdata.generate("dense-lr", n_rows=20, n_cols=1025, k=1025), 2, smem) == "k_sgd_resident"
+    assert [bench.sgd_kernel(tiny, m, smem) for m in (0, 4, -1, -2)] == ["k_sgd_levels", "k_sgd_window", "k_bsp_apply",
+                                                                         "k_sgd_ssp"]
