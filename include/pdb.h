@@ -333,8 +333,10 @@ int pdb_ssp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, cons
  * opts->blocks_per_sm blocks per SM each when that is set (and then no launch
  * overlaps the one before it; 0 = each kernel's own grid).  No kernel waits for
  * another's memory, so opts->wait_timeout_s has nothing to limit.  Allocates
- * per-call scratch stream-ordered and waits (host) for the conflict build of c
- * to finish. */
+ * per-call scratch stream-ordered.  The host waits for the conflict build of c
+ * to finish, and, as for any sequence of launches, while more of them are
+ * pending than the launch queue holds (about a thousand): a call of 2 * batches *
+ * n_epochs launches beyond that returns when all but the last ones have run. */
 int pdb_bsp_epoch(const pdb_csr *X, const float *y, const pdb_conflicts *c, float *w, pdb_loss loss, float eta,
                   int64_t batch, int n_epochs, const pdb_opts *opts, void *stream);
 

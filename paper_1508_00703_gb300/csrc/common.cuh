@@ -24,7 +24,7 @@ struct Launch {
 };
 Launch launch_info();
 int occupancy_blocks(const void *kernel, int threads, size_t smem);
-int persistent_grid(const void *kernel, const pdb_opts *opts, int threads = THREADS);
+int persistent_grid(const void *kernel, const pdb_opts *opts);
 uint64_t timeout_ns(const pdb_opts *opts);
 int alloc(void **p, size_t bytes, cudaStream_t s);   // stream-ordered, 256-byte aligned
 void release(void *p, cudaStream_t s);

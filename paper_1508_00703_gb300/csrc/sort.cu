@@ -28,10 +28,10 @@ int occupancy_blocks(const void *kernel, int threads, size_t smem)
     return nb;
 }
 
-int persistent_grid(const void *kernel, const pdb_opts *opts, int threads)
+int persistent_grid(const void *kernel, const pdb_opts *opts)
 {
     Launch l = launch_info();
-    int nb = occupancy_blocks(kernel, threads, 0);
+    int nb = occupancy_blocks(kernel, THREADS, 0);
     if (opts && opts->blocks_per_sm > 0 && opts->blocks_per_sm < nb) nb = opts->blocks_per_sm;
     if (nb < 1) nb = 1;
     return nb * l.sms;

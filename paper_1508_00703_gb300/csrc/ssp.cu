@@ -86,12 +86,16 @@ __device__ __forceinline__ bool keep_waiting(unsigned &spins, uint64_t t0, int *
 // what a counted access to one word costs here), instead of backing off blindly.
 // Measured, 200k examples of 20 zipf(1.0) ids, delay 1024: doubling naps of up
 // to 512 ns 4.0-6.2 ms over boxes, 4 ns per missing count 3.0, 8 ns 2.2, 12 ns
-// 1.6; the results differ by what two runs of one form differ by (which
-// examples are in flight is the same; fewer warps would be faster still, down to
-// 0.9 ms, with reads less stale).  At small delays few counts are missing but each
-// takes a whole hop: a poll that finds no progress doubles the nap, from 64 to
-// 512 ns (1M such examples, delay 16: doubling alone 783 ms, both 522; delay 128:
-// 154 and 94).
+// 1.6.  Reads get a little less stale: on three Zipf shapes the weights moved by
+// 4e-4 to 1.2e-3 (2-norm) against the blind naps, towards exact SGD (6.0e-3 -> 5.7e-3
+// off, 8.2e-3 -> 7.3e-3), where two runs of one form differ by 1e-4 to 2e-4.  Fewer warps
+// would be faster still, down to 0.9 ms, with reads less stale yet.
+// At small delays few counts are missing but each takes a whole hop: a poll
+// that finds no progress doubles the nap, from 64 to 512 ns.  Measured, one epoch,
+// blind naps / by missing counts alone / with the doubling: 1M such examples, delay 16
+// 654 / 587 / 412 ms, delay 128 156 / 84 / 76; 200k, delay 0 1309 / 1286 / 930; 2M of 200
+// zipf(1.3) ids, delay 1024 279 / 130 / 219 (the doubling costs there), delay 128
+// (200k) 154 / 93 / 110.
 constexpr long long WAIT_NS = 12;
 __device__ __forceinline__ bool wait_count(const unsigned *counter, long long need, int *status, uint64_t timeout)
 {
