@@ -749,7 +749,7 @@ __global__ __launch_bounds__(256, 5) void k_bsp_coef(int64_t r0, int64_t r1, con
 }
 
 // The write half of batch bi: coef holds the whole batch's coefficients (rows
-// r0.. in order).  Long runs one per block; short ones one per thread, on the
+// r0.. in order).  Long runs one per block; short ones BSP_R per thread, on the
 // blocks without a long one when those are most.
 //
 // What bounds it: the longest run's additions (3000 terms of the hottest
